@@ -28,6 +28,18 @@ __device__ __forceinline__ uint32_t x_order_key(float x) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+// Multiply-adds of the half-planes and the LPs, with the rounding fixed: the
+// first product is fused, the second rounded.  The per-thread and the
+// warp-per-agent solve kernels evaluate the same expressions, and a scene's
+// results must not depend on which of them ran, so no contraction is left to
+// the compiler's choice.
+__device__ __forceinline__ float mul_add(float a, float b, float c, float d) {   // a b + c d
+    return __fmaf_rn(a, b, __fmul_rn(c, d));
+}
+__device__ __forceinline__ float mul_sub(float a, float b, float c, float d) {   // a b - c d
+    return __fmaf_rn(a, b, -__fmul_rn(c, d));
+}
+
 // Neighbour key d^2 = fl32(fl32(dx*dx) + fl32(dy*dy)), dx = fl32(xb - xa).
 __device__ __forceinline__ float key_d2(float xa, float ya, float xb, float yb) {
     float dx = __fsub_rn(xb, xa);
@@ -76,7 +88,7 @@ __device__ __forceinline__ bool leg_left(float pax, float pay, float pbx, float 
 // 2^-47 rho^2 (as accurate as an FP64 evaluation, without the FP64 pipe).
 __device__ __forceinline__ float leg_l2(float qx, float qy, float ra, float rb, float qq,
                                         float rho2) {
-    float l2 = qq - rho2;
+    float l2 = __fsub_rn(qq, rho2);
     if (l2 < 0.015625f * qq) {
         // qx^2 = px + ex, qy^2 = py + ey, s^2 = ps + es exactly
         const float px = __fmul_rn(qx, qx), ex = __fmaf_rn(qx, qx, -px);
@@ -113,51 +125,51 @@ __device__ __forceinline__ float4 orca_line(float pax, float pay, float vax, flo
                                             float vby, float rb, float f, float inv_tau,
                                             float inv_dt, bool overlap, bool& cap) {
     cap = false;
-    float qx = pbx - pax, qy = pby - pay;
-    float wrx = vax - vbx, wry = vay - vby;
-    float rho = ra + rb;
+    const float qx = __fsub_rn(pbx, pax), qy = __fsub_rn(pby, pay);
+    const float wrx = __fsub_rn(vax, vbx), wry = __fsub_rn(vay, vby);
+    const float rho = __fadd_rn(ra, rb);
     float ux, uy, dx, dy;
     if (!overlap) {
-        float wx = wrx - qx * inv_tau, wy = wry - qy * inv_tau;
-        float wq = wx * qx + wy * qy;
-        float ww = wx * wx + wy * wy;
-        float rho2 = rho * rho;
-        if (wq < 0.0f && wq * wq > rho2 * ww) {
+        const float wx = __fmaf_rn(-qx, inv_tau, wrx), wy = __fmaf_rn(-qy, inv_tau, wry);
+        const float wq = mul_add(wx, qx, wy, qy);
+        const float ww = mul_add(wx, wx, wy, wy);
+        const float rho2 = __fmul_rn(rho, rho);
+        if (wq < 0.0f && __fmul_rn(wq, wq) > __fmul_rn(rho2, ww)) {
             // cut-off circle
             cap = true;
-            float wl = sqrtf(ww);
-            float hx = wx / wl, hy = wy / wl;
+            const float wl = sqrtf(ww);
+            const float hx = wx / wl, hy = wy / wl;
             dx = hy;
             dy = -hx;
-            float s = rho * inv_tau - wl;
-            ux = s * hx;
-            uy = s * hy;
+            const float s = __fmaf_rn(rho, inv_tau, -wl);
+            ux = __fmul_rn(s, hx);
+            uy = __fmul_rn(s, hy);
         } else {
             // legs
-            float qq = qx * qx + qy * qy;
-            float l = sqrtf(fmaxf(leg_l2(qx, qy, ra, rb, qq, rho2), 0.0f));
-            bool left = leg_left(pax, pay, pbx, pby, vax, vay, vbx, vby);
-            float iq = 1.0f / qq;
+            const float qq = mul_add(qx, qx, qy, qy);
+            const float l = sqrtf(fmaxf(leg_l2(qx, qy, ra, rb, qq, rho2), 0.0f));
+            const bool left = leg_left(pax, pay, pbx, pby, vax, vay, vbx, vby);
+            const float iq = 1.0f / qq;
             if (left) {
-                dx = (qx * l - qy * rho) * iq;
-                dy = (qx * rho + qy * l) * iq;
+                dx = __fmul_rn(mul_sub(qx, l, qy, rho), iq);
+                dy = __fmul_rn(mul_add(qx, rho, qy, l), iq);
             } else {
-                dx = -(qx * l + qy * rho) * iq;
-                dy = -(qy * l - qx * rho) * iq;
+                dx = __fmul_rn(-mul_add(qy, rho, qx, l), iq);
+                dy = __fmul_rn(-mul_sub(qy, l, qx, rho), iq);
             }
-            float pr = wrx * dx + wry * dy;
-            ux = pr * dx - wrx;
-            uy = pr * dy - wry;
+            const float pr = mul_add(wrx, dx, wry, dy);
+            ux = __fmaf_rn(pr, dx, -wrx);
+            uy = __fmaf_rn(pr, dy, -wry);
         }
     } else {
-        float wx = wrx - qx * inv_dt, wy = wry - qy * inv_dt;
-        float wl = sqrtf(wx * wx + wy * wy);
+        const float wx = __fmaf_rn(-qx, inv_dt, wrx), wy = __fmaf_rn(-qy, inv_dt, wry);
+        const float wl = sqrtf(mul_add(wx, wx, wy, wy));
         float hx, hy;
         if (wl > 0.0f) {
             hx = wx / wl;
             hy = wy / wl;
         } else {
-            float ql = sqrtf(qx * qx + qy * qy);
+            const float ql = sqrtf(mul_add(qx, qx, qy, qy));
             if (ql > 0.0f) {
                 hx = -qx / ql;
                 hy = -qy / ql;
@@ -168,16 +180,16 @@ __device__ __forceinline__ float4 orca_line(float pax, float pay, float vax, flo
         }
         dx = hy;
         dy = -hx;
-        float s = rho * inv_dt - wl;
-        ux = s * hx;
-        uy = s * hy;
+        const float s = __fmaf_rn(rho, inv_dt, -wl);
+        ux = __fmul_rn(s, hx);
+        uy = __fmul_rn(s, hy);
     }
-    return make_float4(vax + f * ux, vay + f * uy, dx, dy);
+    return make_float4(__fmaf_rn(f, ux, vax), __fmaf_rn(f, uy, vay), dx, dy);
 }
 
 // det(d, P - v): positive = v violates the half-plane
 __device__ __forceinline__ float penetration(float4 L, float vx, float vy) {
-    return L.z * (L.y - vy) - L.w * (L.x - vx);
+    return mul_sub(L.z, __fsub_rn(L.y, vy), L.w, __fsub_rn(L.x, vx));
 }
 
 // ---------------------------------------------------------------------------
@@ -228,7 +240,55 @@ __host__ __device__ __forceinline__ bool act_overlap(uint32_t a, int m) {
 // of f = 0 pairs all pass through the agent's own velocity, and when that
 // lies on the speed circle their exact common point meets the circle's
 // rounded end (a vehicle at full speed among pedestrians).
-__device__ __forceinline__ float lp_tol(float vmax) { return 1e-5f * (1.0f + vmax); }
+__device__ __forceinline__ float lp_tol(float vmax) {
+    return __fmul_rn(1e-5f, __fadd_rn(1.0f, vmax));
+}
+
+// The interval [tl, tr] of the line p + t d (unit d) inside the disc |v| <= vmax;
+// false when the line misses it by more than the rounding allowance.
+__device__ __forceinline__ bool disc_chord(float px, float py, float dx, float dy, float vmax,
+                                           float tol, float& tl, float& tr) {
+    const float dot = mul_add(px, dx, py, dy);
+    const float disc = __fsub_rn(mul_add(dot, dot, vmax, vmax), mul_add(px, px, py, py));
+    if (disc < -tol * (1.0f + vmax)) return false;
+    const float sq = sqrtf(fmaxf(disc, 0.0f));
+    tl = __fsub_rn(-dot, sq);
+    tr = __fadd_rn(-dot, sq);
+    return true;
+}
+
+// Bound that half-plane j puts on the parameter t of line i: t <= num / den
+// for den > 0, t >= num / den for den < 0 (den = 0: parallel lines, line i
+// inside half-plane j when num >= 0).
+__device__ __forceinline__ void line_bound(float4 li, float4 lj, float& den, float& num) {
+    den = mul_sub(li.z, lj.w, li.w, lj.z);                                            // det(d_i, d_j)
+    num = mul_sub(lj.z, __fsub_rn(li.y, lj.y), lj.w, __fsub_rn(li.x, lj.x));   // det(d_j, P_i - P_j)
+}
+
+// Point of line i at the parameter in [tl, tr] closest to v_pref; returns the
+// unclamped parameter.
+__device__ __forceinline__ float line_project(float4 li, float vpx, float vpy, float tl, float tr,
+                                              float& ox, float& oy) {
+    const float t0 = mul_add(li.z, __fsub_rn(vpx, li.x), li.w, __fsub_rn(vpy, li.y));
+    const float t = fminf(fmaxf(t0, tl), tr);
+    ox = __fmaf_rn(t, li.z, li.x);
+    oy = __fmaf_rn(t, li.w, li.y);
+    return t0;
+}
+
+// v_pref, capped to the speed disc: the 2D LP's start.  Returns whether the
+// cap took effect.
+__device__ __forceinline__ bool disc_project(float vmax, float vpx, float vpy, float& vx,
+                                             float& vy) {
+    const float vp2 = mul_add(vpx, vpx, vpy, vpy);
+    vx = vpx;
+    vy = vpy;
+    if (!(vp2 > __fmul_rn(vmax, vmax))) return false;
+    const float s = vmax / sqrtf(vp2);
+    vx = __fmul_rn(vpx, s);
+    vy = __fmul_rn(vpy, s);
+    return true;
+}
 
 // 1D problem on line i: the point of line i closest to v_pref that keeps
 // lines 0..i-1 and the disc.  Returns false when that set is empty.
@@ -237,24 +297,20 @@ __device__ __forceinline__ float lp_tol(float vmax) { return 1e-5f * (1.0f + vma
 __device__ __forceinline__ bool lp1_project(const float4* __restrict__ L, int stride, int i,
                                             float vmax, float vpx, float vpy, float& ox,
                                             float& oy, int& work, int& bound) {
-    float4 li = L[i * stride];
+    const float4 li = L[i * stride];
     const float tol = lp_tol(vmax);
-    float dot = li.x * li.z + li.y * li.w;
-    float disc = dot * dot + vmax * vmax - (li.x * li.x + li.y * li.y);
-    if (disc < -tol * (1.0f + vmax)) return false;
-    float sq = sqrtf(fmaxf(disc, 0.0f));
-    float tl = -dot - sq, tr = -dot + sq;
+    float tl, tr;
+    if (!disc_chord(li.x, li.y, li.z, li.w, vmax, tol, tl, tr)) return false;
     int jl = -1, jr = -1;
     for (int j = 0; j < i; ++j) {
         ++work;
-        float4 lj = L[j * stride];
-        float den = li.z * lj.w - li.w * lj.z;                     // det(d_i, d_j)
-        float num = lj.z * (li.y - lj.y) - lj.w * (li.x - lj.x);   // det(d_j, P_i - P_j)
+        float den, num;
+        line_bound(li, L[j * stride], den, num);
         if (den == 0.0f) {
             if (num < -tol) return false;
             continue;
         }
-        float t = __fdividef(num, den);
+        const float t = __fdividef(num, den);
         if (den > 0.0f) {
             if (t < tr) jr = j;
             tr = fminf(tr, t);
@@ -264,11 +320,8 @@ __device__ __forceinline__ bool lp1_project(const float4* __restrict__ L, int st
         }
         if (tl > tr + tol) return false;
     }
-    float t0 = li.z * (vpx - li.x) + li.w * (vpy - li.y);
-    float t = fminf(fmaxf(t0, tl), tr);
+    const float t0 = line_project(li, vpx, vpy, tl, tr, ox, oy);
     bound = (t0 > tr) ? jr : ((t0 < tl) ? jl : -2);
-    ox = li.x + t * li.z;
-    oy = li.y + t * li.w;
     return true;
 }
 
@@ -278,17 +331,8 @@ __device__ __forceinline__ bool lp1_project(const float4* __restrict__ L, int st
 __device__ __forceinline__ int lp2_project(const float4* __restrict__ L, int stride, int n,
                                            float vmax, float vpx, float vpy, float& vx,
                                            float& vy, int& work, uint32_t& act) {
-    float vp2 = vpx * vpx + vpy * vpy;
-    if (vp2 > vmax * vmax) {
-        float s = vmax / sqrtf(vp2);
-        vx = vpx * s;
-        vy = vpy * s;
-        act = act_pack(ACT_PROJ, true, 0, 0, 0, 0);
-    } else {
-        vx = vpx;
-        vy = vpy;
-        act = act_pack(ACT_PROJ, false, 0, 0, 0, 0);
-    }
+    const bool capped = disc_project(vmax, vpx, vpy, vx, vy);
+    act = act_pack(ACT_PROJ, capped, 0, 0, 0, 0);
     for (int i = 0; i < n; ++i) {
         float4 li = L[i * stride];
         if (penetration(li, vx, vy) > 0.0f) {
@@ -312,15 +356,15 @@ __device__ __forceinline__ int lp2_project(const float4* __restrict__ L, int str
 // opposite lines and lose all FP32 precision).  Returns false for parallel
 // lines of the same direction (one of them dominates everywhere).
 __device__ __forceinline__ bool bisector(float4 li, float4 lj, float4& b) {
-    const float ax = li.w - lj.w;          // n_j - n_i, n = (-d_y, d_x)
-    const float ay = lj.z - li.z;
-    const float a2 = ax * ax + ay * ay;
+    const float ax = __fsub_rn(li.w, lj.w);          // n_j - n_i, n = (-d_y, d_x)
+    const float ay = __fsub_rn(lj.z, li.z);
+    const float a2 = mul_add(ay, ay, ax, ax);
     if (a2 <= 1e-12f) return false;
-    const float ci = li.z * li.y - li.w * li.x;
-    const float cj = lj.z * lj.y - lj.w * lj.x;
-    const float s = __fdividef(cj - ci, a2);
+    const float ci = mul_sub(li.z, li.y, li.w, li.x);
+    const float cj = mul_sub(lj.z, lj.y, lj.w, lj.x);
+    const float s = __fdividef(__fsub_rn(cj, ci), a2);
     const float inv = rsqrtf(a2);
-    b = make_float4(ax * s, ay * s, ay * inv, -ax * inv);
+    b = make_float4(__fmul_rn(ax, s), __fmul_rn(ay, s), __fmul_rn(ay, inv), -__fmul_rn(ax, inv));
     return true;
 }
 
@@ -340,63 +384,94 @@ __device__ __forceinline__ bool bisector(float4 li, float4 lj, float4& b) {
 // look empty (a bisector that misses the disc, or a 1D interval emptier than
 // the allowance) the step keeps its current point, and *fallback is set: the
 // result is then only an upper bound of t*.
+
+// Plane j against plane i: a = n_j - n_i, |a|^2 and beta = c'_j - c'_i
+// (ci, cj: det(d, P - s) of the two, from penetration()).
+struct PlanePair {
+    float ax, ay, a2, beta;
+};
+__device__ __forceinline__ PlanePair plane_pair(float4 li, float ci, float4 lj, float cj) {
+    PlanePair q;
+    q.ax = __fsub_rn(li.w, lj.w);
+    q.ay = __fsub_rn(lj.z, li.z);
+    q.a2 = mul_add(q.ay, q.ay, q.ax, q.ax);
+    q.beta = __fsub_rn(cj, ci);
+    return q;
+}
+
+// Whether plane j lies above plane i at c: (n_j - n_i) . (c - s) < c'_j - c'_i.
+__device__ __forceinline__ bool plane_above(const PlanePair& q, float cx, float cy, float sx,
+                                            float sy) {
+    const float d = mul_add(q.ax, __fsub_rn(cx, sx), q.ay, __fsub_rn(cy, sy));
+    return !(__fsub_rn(q.beta, d) <= 0.0f);
+}
+
+// The bisector {det_j = det_i}, (n_j - n_i) . (v - s) = c'_j - c'_i, as a line
+// through its point closest to s (B' relative to s, B in ordinary
+// coordinates) with unit direction e, the side det_j <= det_i on its left.
+struct PairLine {
+    float bpx, bpy, bx, by, ex, ey;
+};
+__device__ __forceinline__ PairLine pair_line(const PlanePair& q, float sx, float sy) {
+    const float sc = __fdividef(q.beta, q.a2);
+    const float inv = rsqrtf(q.a2);
+    PairLine b;
+    b.bpx = __fmul_rn(q.ax, sc);
+    b.bpy = __fmul_rn(q.ay, sc);
+    b.ex = __fmul_rn(q.ay, inv);
+    b.ey = -__fmul_rn(q.ax, inv);
+    b.bx = __fadd_rn(b.bpx, sx);
+    b.by = __fadd_rn(b.bpy, sy);
+    return b;
+}
+
+// Plane jj stays below plane i along the bisector s + B' + t e:
+// t (a . e) >= beta - a . B'.
+__device__ __forceinline__ void pair_bound(const PlanePair& q, const PairLine& b, float& den,
+                                           float& num) {
+    den = mul_add(q.ay, b.ey, q.ax, b.ex);
+    num = __fsub_rn(q.beta, mul_add(q.ay, b.bpy, q.ax, b.bpx));
+}
+
 __device__ __forceinline__ float lp3_min_penetration(const float4* __restrict__ L, int stride,
                                                      int n, float vmax, float sx, float sy,
                                                      float& vx, float& vy, int& work,
                                                      uint32_t& act, bool* fallback = nullptr) {
     const float tol = lp_tol(vmax);
-    // det(d, P - s)
-    auto cof = [&](float4 l) { return l.z * (l.y - sy) - l.w * (l.x - sx); };
     float4 l0 = L[0];
-    vx = -l0.w * vmax;
-    vy = l0.z * vmax;
+    vx = __fmul_rn(-l0.w, vmax);
+    vy = __fmul_rn(l0.z, vmax);
     act = act_pack(ACT_VERTEX, true, 1, 0, 0, 0);
     float t = penetration(l0, vx, vy);
     for (int i = 1; i < n; ++i) {
-        float4 li = L[i * stride];
+        const float4 li = L[i * stride];
         if (penetration(li, vx, vy) <= t) continue;
-        float nix = -li.w, niy = li.z;   // objective: maximise n_i . v
-        float cx = vmax * nix, cy = vmax * niy;
-        const float ci = cof(li);
+        const float nix = -li.w, niy = li.z;   // objective: maximise n_i . v
+        float cx = __fmul_rn(vmax, nix), cy = __fmul_rn(vmax, niy);
+        const float ci = penetration(li, sx, sy);   // det(d, P - s)
         uint32_t ai = act_pack(ACT_VERTEX, true, 1, i, 0, 0);
         for (int j = 0; j < i; ++j) {
             ++work;
             const float4 lj = L[j * stride];
-            // is plane j above plane i at the current point?
-            // (n_j - n_i) . (c - s) < c'_j - c'_i, tested before the bisector is built
-            const float ax = li.w - lj.w, ay = lj.z - li.z;   // n_j - n_i
-            const float beta = cof(lj) - ci;
-            if (beta - (ax * (cx - sx) + ay * (cy - sy)) <= 0.0f) continue;
-            // bisector {det_j = det_i}: (n_j - n_i) . (v - s) = c'_j - c'_i, as a
-            // line through its point closest to s, B' relative to s, with
-            // direction e (admissible side det_j <= det_i on its left)
-            const float a2 = ax * ax + ay * ay;
-            if (a2 <= 1e-12f) continue;   // same direction: one plane dominates
-            const float sc = __fdividef(beta, a2);
-            const float inv = rsqrtf(a2);
-            const float bpx = ax * sc, bpy = ay * sc;
-            const float ex = ay * inv, ey = -ax * inv;
-            const float bx = bpx + sx, by = bpy + sy;
-            float dot = bx * ex + by * ey;
-            float disc = dot * dot + vmax * vmax - (bx * bx + by * by);
-            if (disc < -tol * (1.0f + vmax)) {
+            const PlanePair q = plane_pair(li, ci, lj, penetration(lj, sx, sy));
+            // tested before the bisector is built
+            if (!plane_above(q, cx, cy, sx, sy)) continue;
+            if (q.a2 <= 1e-12f) continue;   // same direction: one plane dominates
+            const PairLine b = pair_line(q, sx, sy);
+            float tl, tr;
+            if (!disc_chord(b.bx, b.by, b.ex, b.ey, vmax, tol, tl, tr)) {
                 if (fallback) *fallback = true;
                 continue;
             }
-            float sq = sqrtf(fmaxf(disc, 0.0f));
-            float tl = -dot - sq, tr = -dot + sq;
             int kl = -1, kr = -1;
             bool ok = true;
             for (int jj = 0; jj < j; ++jj) {
                 work += 2;   // a bisector and a 1D bound
-                // plane jj stays below plane i: (n_jj - n_i) . (v - s) >= c'_jj - c'_i,
-                // on the bisector at v = s + B' + t e: t (a . e) >= (c'_jj - c'_i) - a . B'
                 const float4 lk = L[jj * stride];
-                const float kx = li.w - lk.w, ky = lk.z - li.z;   // n_jj - n_i
-                if (kx * kx + ky * ky <= 1e-12f) continue;        // same direction
-                const float bk = cof(lk) - ci;
-                const float den = kx * ex + ky * ey;
-                const float num = bk - (kx * bpx + ky * bpy);
+                const PlanePair k = plane_pair(li, ci, lk, penetration(lk, sx, sy));
+                if (k.a2 <= 1e-12f) continue;        // same direction
+                float den, num;
+                pair_bound(k, b, den, num);
                 if (den == 0.0f) {
                     if (num > tol) { ok = false; break; }
                     continue;
@@ -415,11 +490,11 @@ __device__ __forceinline__ float lp3_min_penetration(const float4* __restrict__ 
                 if (fallback) *fallback = true;
                 continue;
             }
-            const bool right = nix * ex + niy * ey > 0.0f;
-            float tt = right ? tr : tl;
+            const bool right = mul_add(nix, b.ex, niy, b.ey) > 0.0f;
+            const float tt = right ? tr : tl;
             const int kb = right ? kr : kl;
-            cx = bx + tt * ex;
-            cy = by + tt * ey;
+            cx = __fmaf_rn(tt, b.ex, b.bx);
+            cy = __fmaf_rn(tt, b.ey, b.by);
             ai = kb >= 0 ? act_pack(ACT_VERTEX, false, 3, i, j, kb)
                          : act_pack(ACT_VERTEX, true, 2, i, j, 0);
         }
@@ -433,54 +508,27 @@ __device__ __forceinline__ float lp3_min_penetration(const float4* __restrict__ 
     return tm;
 }
 
-// The set of least-penetration velocities is one point unless two of the
-// half-planes attaining t* are exactly opposite (a valley between two
-// neighbours); then it is the part of the valley's mid-line that keeps every
-// other half-plane within t* and the disc, and the result is its point
-// closest to v_pref.  Returns true and writes that point for a valley.
-__device__ __forceinline__ bool valley_tie_break(const float4* __restrict__ L, int stride,
-                                                 int n, float t3, float vmax, float vpx,
-                                                 float vpy, float v3x, float v3y, float& ox,
-                                                 float& oy, int& work, uint32_t& act) {
-    const float atol = 1e-5f * (1.0f + fabsf(t3));
-    // the lines attaining t* (within atol), then the first exactly opposite
-    // pair among them, in the order (i, j) of the line indices
-    unsigned long long amask = 0ull;
-    for (int i = 0; i < n; ++i)
-        if (!(penetration(L[i * stride], v3x, v3y) < t3 - atol)) amask |= 1ull << i;
-    int vi = -1, vj = -1;
-    for (unsigned long long m = amask; m != 0ull && vi < 0; m &= m - 1ull) {
-        const int i = __ffsll((long long)m) - 1;
-        const float4 li = L[i * stride];
-        for (unsigned long long m2 = m & (m - 1ull); m2 != 0ull; m2 &= m2 - 1ull) {
-            const int j = __ffsll((long long)m2) - 1;
-            ++work;
-            const float4 lj = L[j * stride];
-            if (fabsf(li.z * lj.w - li.w * lj.z) > 2e-7f || li.z * lj.z + li.w * lj.w >= 0.0f)
-                continue;
-            vi = i;
-            vj = j;
-            break;
-        }
-    }
-    if (vi < 0) return false;
+// The point closest to v_pref on the mid-line of the two exactly opposite
+// half-planes vi and vj that keeps every other half-plane within t3 and the
+// disc; false when there is none.
+__device__ __forceinline__ bool valley_project(const float4* __restrict__ L, int stride, int n,
+                                               int vi, int vj, float t3, float vmax, float vpx,
+                                               float vpy, float& ox, float& oy, int& work,
+                                               uint32_t& act) {
     float4 m;
     if (!bisector(L[vi * stride], L[vj * stride], m)) return false;
     const float tol = lp_tol(vmax);
-    const float dot = m.x * m.z + m.y * m.w;
-    const float disc = dot * dot + vmax * vmax - (m.x * m.x + m.y * m.y);
-    if (disc < -tol * (1.0f + vmax)) return false;
-    const float sq = sqrtf(fmaxf(disc, 0.0f));
-    float tl = -dot - sq, tr = -dot + sq;
-    const float T = t3 + 1e-6f * (1.0f + fabsf(t3));
+    float tl, tr;
+    if (!disc_chord(m.x, m.y, m.z, m.w, vmax, tol, tl, tr)) return false;
+    const float T = __fmaf_rn(1e-6f, 1.0f + fabsf(t3), t3);
     int kl = -1, kr = -1;
     for (int k = 0; k < n; ++k) {
         if (k == vi || k == vj) continue;
         ++work;
         const float4 lk = L[k * stride];
         // det(d_k, P_k - (M + s e)) <= T  <=>  s det(e, d_k) <= T - det(d_k, P_k - M)
-        const float den = m.z * lk.w - m.w * lk.z;
-        const float num = T - (lk.z * (lk.y - m.y) - lk.w * (lk.x - m.x));
+        const float den = mul_sub(m.z, lk.w, m.w, lk.z);
+        const float num = __fsub_rn(T, penetration(lk, m.x, m.y));
         if (den == 0.0f) {
             if (num < -tol) return false;
             continue;
@@ -495,15 +543,56 @@ __device__ __forceinline__ bool valley_tie_break(const float4* __restrict__ L, i
         }
     }
     if (tl > tr + tol) return false;
-    const float s0 = m.z * (vpx - m.x) + m.w * (vpy - m.y);
-    const float s = fminf(fmaxf(s0, tl), tr);
+    const float s0 = line_project(m, vpx, vpy, tl, tr, ox, oy);
     const int kb = (s0 > tr) ? kr : ((s0 < tl) ? kl : -2);
     act = kb >= 0   ? act_pack(ACT_VERTEX, false, 3, vi, vj, kb)
           : kb == -1 ? act_pack(ACT_VERTEX, true, 2, vi, vj, 0)
                      : act_pack(ACT_VALLEY, false, 2, vi, vj, 0);
-    ox = m.x + s * m.z;
-    oy = m.y + s * m.w;
     return true;
+}
+
+// A line attains the least penetration t3 when its own is not below this.
+__device__ __forceinline__ float attains_limit(float t3) {
+    return __fmaf_rn(-1e-5f, __fadd_rn(1.0f, fabsf(t3)), t3);
+}
+
+// Whether two of the lines that attain t* are exactly opposite.
+__device__ __forceinline__ bool opposite(float4 li, float4 lj) {
+    return !(fabsf(mul_sub(li.z, lj.w, li.w, lj.z)) > 2e-7f ||
+             mul_add(li.z, lj.z, li.w, lj.w) >= 0.0f);
+}
+
+// The set of least-penetration velocities is one point unless two of the
+// half-planes attaining t* are exactly opposite (a valley between two
+// neighbours); then it is the part of the valley's mid-line that keeps every
+// other half-plane within t* and the disc, and the result is its point
+// closest to v_pref.  Returns true and writes that point for a valley.
+__device__ __forceinline__ bool valley_tie_break(const float4* __restrict__ L, int stride,
+                                                 int n, float t3, float vmax, float vpx,
+                                                 float vpy, float v3x, float v3y, float& ox,
+                                                 float& oy, int& work, uint32_t& act) {
+    const float tmin = attains_limit(t3);
+    // the lines attaining t* (within atol), then the first exactly opposite
+    // pair among them, in the order (i, j) of the line indices
+    unsigned long long amask = 0ull;
+    for (int i = 0; i < n; ++i)
+        if (!(penetration(L[i * stride], v3x, v3y) < tmin)) amask |= 1ull << i;
+    int vi = -1, vj = -1;
+    for (unsigned long long m = amask; m != 0ull && vi < 0; m &= m - 1ull) {
+        const int i = __ffsll((long long)m) - 1;
+        const float4 li = L[i * stride];
+        for (unsigned long long m2 = m & (m - 1ull); m2 != 0ull; m2 &= m2 - 1ull) {
+            const int j = __ffsll((long long)m2) - 1;
+            ++work;
+            const float4 lj = L[j * stride];
+            if (!opposite(li, lj)) continue;
+            vi = i;
+            vj = j;
+            break;
+        }
+    }
+    if (vi < 0) return false;
+    return valley_project(L, stride, n, vi, vj, t3, vmax, vpx, vpy, ox, oy, work, act);
 }
 
 // The velocity of one agent (paper Sec. 3): the admissible velocity closest
@@ -691,6 +780,21 @@ __device__ __forceinline__ int solve_velocity_work_units(const float4* __restric
 //   valley tie-break.
 // O(k^3) work per agent, against O(k^2) for the incremental scheme.
 // ---------------------------------------------------------------------------
+// The bisector of two lines as the comparison schemes build it (rounding left
+// to the compiler's contraction).
+__device__ __forceinline__ bool plain_bisector(float4 li, float4 lj, float4& b) {
+    const float ax = li.w - lj.w;
+    const float ay = lj.z - li.z;
+    const float a2 = ax * ax + ay * ay;
+    if (a2 <= 1e-12f) return false;
+    const float ci = li.z * li.y - li.w * li.x;
+    const float cj = lj.z * lj.y - lj.w * lj.x;
+    const float s = __fdividef(cj - ci, a2);
+    const float inv = rsqrtf(a2);
+    b = make_float4(ax * s, ay * s, ay * inv, -ax * inv);
+    return true;
+}
+
 __device__ __forceinline__ float max_penetration(const float4* __restrict__ L, int stride, int n,
                                                  float x, float y) {
     float t = -CUDART_INF_F;
@@ -771,7 +875,7 @@ __device__ __forceinline__ int solve_velocity_enumeration(const float4* __restri
         for (int j = 0; j < i; ++j) {
             const float4 lj = L[j * stride];
             float4 bij;
-            if (!bisector(li, lj, bij)) continue;
+            if (!plain_bisector(li, lj, bij)) continue;
             const float dot = bij.x * bij.z + bij.y * bij.w;
             const float disc = dot * dot + vmax * vmax - (bij.x * bij.x + bij.y * bij.y);
             if (disc >= 0.0f) {
@@ -922,7 +1026,7 @@ __device__ __forceinline__ int solve_velocity_warp(const float4* __restrict__ li
                         if (beta - (ax * cx + ay * cy) <= 0.0f) continue;
                     }
                     float4 bj;
-                    if (!bisector(li, lj, bj)) continue;
+                    if (!plain_bisector(li, lj, bj)) continue;
                     const float dot = bj.x * bj.z + bj.y * bj.w;
                     const float disc = dot * dot + vmax * vmax - (bj.x * bj.x + bj.y * bj.y);
                     if (disc < -tol * (1.0f + vmax)) continue;

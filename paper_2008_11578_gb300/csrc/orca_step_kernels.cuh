@@ -585,6 +585,75 @@ __global__ void compact_scatter_kernel(int kept, const float2* __restrict__ t_po
     if (kept_index != nullptr) kept_index[d] = (int32_t)t_orig[d].x;
 }
 
+// ------------------------------------------- pieces of the solve kernels ----
+// Shared by the per-thread and the warp-per-agent solve kernels, with the
+// rounding fixed (see mul_add): a step's results do not depend on which ran.
+
+// Preferred velocity toward target g: maximum speed, capped so as not to
+// overshoot within the step, plus the caller's offset.
+__device__ __forceinline__ float2 preferred_velocity(float2 p, float2 g, float vmax, float inv_dt,
+                                                     bool offset, float2 dl) {
+    const float gx = __fsub_rn(g.x, p.x), gy = __fsub_rn(g.y, p.y);
+    const float gl = sqrtf(mul_add(gx, gx, gy, gy));
+    float2 w = make_float2(0.0f, 0.0f);
+    if (gl > 0.0f) {
+        const float f = fminf(vmax / gl, inv_dt);
+        w = make_float2(__fmul_rn(gx, f), __fmul_rn(gy, f));
+    }
+    if (offset) {
+        w.x = __fadd_rn(w.x, dl.x);
+        w.y = __fadd_rn(w.y, dl.y);
+    }
+    return w;
+}
+
+// The waypoint a routed agent heads for, advanced when it is within the
+// agent's radius: its index after the step, and its position in g.
+__device__ __forceinline__ int advance_waypoint(const float2* __restrict__ W, int n_waypoints,
+                                                int wi, float2 p, float r, float2& g) {
+    const float2 w = W[wi];
+    const float wdx = __fsub_rn(w.x, p.x), wdy = __fsub_rn(w.y, p.y);
+    const float w2 = __fadd_rn(__fmul_rn(wdx, wdx), __fmul_rn(wdy, wdy));
+    if (wi < n_waypoints - 1 && w2 <= __fmul_rn(r, r)) ++wi;
+    g = W[wi];
+    return wi;
+}
+
+// Half-planes of a vehicle's kinematic limits (at most kKinLines), appended
+// through put(line).
+template <class PUT>
+__device__ __forceinline__ void limit_lines(const SceneDev& sc, float2 v, float2 vp, PUT put) {
+    const float sp2 = __fadd_rn(__fmul_rn(v.x, v.x), __fmul_rn(v.y, v.y));
+    const bool moving = sp2 >= 0.01f;   // |v| >= 0.1 m/s: the heading is defined
+    float hx = 0.0f, hy = 0.0f, sp = 0.0f;
+    if (moving) {
+        sp = sqrtf(sp2);
+        hx = v.x / sp;
+        hy = v.y / sp;
+    } else {
+        const float pl = sqrtf(mul_add(vp.x, vp.x, vp.y, vp.y));
+        if (pl > 0.0f) {
+            hx = vp.x / pl;
+            hy = vp.y / pl;
+        }
+    }
+    if (moving && sc.kin_turn) {
+        // the heading may turn by at most +-theta: the wedge between the
+        // rays R(+theta) h and R(-theta) h, two half-planes through 0
+        const float lx = mul_sub(sc.cos_turn, hx, sc.sin_turn, hy);
+        const float ly = mul_add(sc.sin_turn, hx, sc.cos_turn, hy);
+        put(make_float4(0.0f, 0.0f, -lx, -ly));
+        const float rx = mul_add(sc.cos_turn, hx, sc.sin_turn, hy);
+        const float ry = -mul_sub(sc.sin_turn, hx, sc.cos_turn, hy);
+        put(make_float4(0.0f, 0.0f, rx, ry));
+    }
+    if (sc.kin_accel && (hx != 0.0f || hy != 0.0f)) {
+        // forward speed gain at most accel * dt: v . h <= |v| + accel dt
+        const float smax = __fadd_rn(sp, sc.accel_dt);
+        put(make_float4(__fmul_rn(smax, hx), __fmul_rn(smax, hy), -hy, hx));
+    }
+}
+
 // ----------------------------------------------------------------- solve ----
 // One thread per agent (sorted slot s).  The neighbour list and then the
 // lines are kept in dynamic shared memory (k float4 slots per thread), slot i
@@ -857,32 +926,16 @@ solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* __res
             }
             if (active && dbg.swp != nullptr) dbg.swp[o] = (uint8_t)wi;
             const float2* W = ain.waypoints + (size_t)rt * ain.n_waypoints;
-            float2 w = W[wi];
-            float wdx = __fsub_rn(w.x, p.x), wdy = __fsub_rn(w.y, p.y);
-            float w2 = __fadd_rn(__fmul_rn(wdx, wdx), __fmul_rn(wdy, wdy));
-            if (wi < ain.n_waypoints - 1 && w2 <= __fmul_rn(r, r)) ++wi;
-            g = W[wi];
+            wi = advance_waypoint(W, ain.n_waypoints, wi, p, r, g);
             if (active) {
                 ain.wp_idx[o] = (uint8_t)wi;
                 if (dbg.wp_used != nullptr) dbg.wp_used[o] = (uint8_t)wi;
             }
         }
     }
-    float vpx = 0.0f, vpy = 0.0f;
-    {
-        float gx = g.x - p.x, gy = g.y - p.y;
-        float gl = sqrtf(gx * gx + gy * gy);
-        if (gl > 0.0f) {
-            float f = fminf(vmax / gl, sc.inv_dt);
-            vpx = gx * f;
-            vpy = gy * f;
-        }
-        if (vpd != nullptr) {
-            float2 dl = vpd[o];
-            vpx += dl.x;
-            vpy += dl.y;
-        }
-    }
+    const float2 vp = preferred_velocity(p, g, vmax, sc.inv_dt, vpd != nullptr,
+                                         vpd != nullptr ? vpd[o] : make_float2(0.0f, 0.0f));
+    const float vpx = vp.x, vpy = vp.y;
 
     // ---- one ORCA half-plane per neighbour (Sec. 3.1) ----
     // Constraint m is the m-th nearest; its line replaces its list entry.
@@ -915,37 +968,8 @@ solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* __res
 
     // ---- vehicles' kinematic half-planes (off unless the scene sets limits) ----
     int nlines = cnt;
-    if (ta != 0 && (sc.kin_turn || sc.kin_accel)) {
-        const float sp2 = __fadd_rn(__fmul_rn(v.x, v.x), __fmul_rn(v.y, v.y));
-        const bool moving = sp2 >= 0.01f;   // |v| >= 0.1 m/s: the heading is defined
-        float hx = 0.0f, hy = 0.0f, sp = 0.0f;
-        if (moving) {
-            sp = sqrtf(sp2);
-            hx = v.x / sp;
-            hy = v.y / sp;
-        } else {
-            const float pl = sqrtf(vpx * vpx + vpy * vpy);
-            if (pl > 0.0f) {
-                hx = vpx / pl;
-                hy = vpy / pl;
-            }
-        }
-        if (moving && sc.kin_turn) {
-            // the heading may turn by at most +-theta: the wedge between the
-            // rays R(+theta) h and R(-theta) h, two half-planes through 0
-            const float lx = sc.cos_turn * hx - sc.sin_turn * hy;
-            const float ly = sc.sin_turn * hx + sc.cos_turn * hy;
-            L[nlines++ * stride] = make_float4(0.0f, 0.0f, -lx, -ly);
-            const float rx = sc.cos_turn * hx + sc.sin_turn * hy;
-            const float ry = -sc.sin_turn * hx + sc.cos_turn * hy;
-            L[nlines++ * stride] = make_float4(0.0f, 0.0f, rx, ry);
-        }
-        if (sc.kin_accel && (hx != 0.0f || hy != 0.0f)) {
-            // forward speed gain at most accel * dt: v . h <= |v| + accel dt
-            const float smax = sp + sc.accel_dt;
-            L[nlines++ * stride] = make_float4(smax * hx, smax * hy, -hy, hx);
-        }
-    }
+    if (ta != 0 && (sc.kin_turn || sc.kin_accel))
+        limit_lines(sc, v, vp, [&](float4 l) { L[nlines++ * stride] = l; });
 
     // ---- constraint order of the LP ----
     // Half-planes in decreasing penetration at the agent's current velocity:
