@@ -25,6 +25,7 @@
 #include "orca.h"
 #include "orca_adjoint.cuh"
 #include "orca_step_kernels.cuh"
+#include "orca_warp_solve.cuh"
 
 using namespace orca;
 
@@ -305,6 +306,19 @@ int step_mode(const Pipeline& P) {
     return (P.flags & ORCA_FLAG_LP_ENUMERATION) ? MODE_ENUMERATION : MODE_PLAIN;
 }
 
+// Largest scene solved with one warp per agent.  One thread per agent takes
+// the length of a thread's serial chain however few agents there are (51 us a
+// launch at 1k to 16k agents with k = 10, 217-233 us with k = 32); a warp's
+// chain is 14 us (45 us at 8k agents with k = 32), but the warps of a larger
+// scene queue (2.2 ns an agent with k = 10, 4.2 with k = 32).  The two meet
+// near 22,000 and 55,000 agents (at 24,000: 57 us against 55 us).
+constexpr int kWarpSolveMax = 20480, kWarpSolveMaxWide = 49152;   // up to 16 lines, more
+
+bool solve_by_warp(const Pipeline& P, int mode) {
+    return (mode == MODE_PLAIN || mode == MODE_RECORD) && P.kcap <= 32 &&
+           P.n <= (P.kcap <= 16 ? kWarpSolveMax : kWarpSolveMaxWide);
+}
+
 // The binning kernel of one step (cooperative launch, grid sized to what is
 // resident at once on this device).  first: from the caller's arrays.
 template <class SRC>
@@ -347,6 +361,8 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
     const int sb = P.block;
     const int sgrid = (n + sb - 1) / sb;
     const size_t smem = solve_smem(P);
+    const bool by_warp = solve_by_warp(P, mode);
+    const int wgrid = (int)(((long long)n * 32 + sb - 1) / sb);
     // NVTX ranges (host side: the enqueue of each step and its two kernels)
     nvtxRangePushA("orca_step");
     for (int t = 0; t < n_steps; ++t) {
@@ -367,8 +383,15 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
                                            nullptr, B.hint, B.err + 1}
                                  : StepOut{B.pos0, B.vel0, false, B.key, B.slot, B.count,
                                            nullptr, nullptr};
-        launch_solve(mode, sgrid, sb, smem, st, n, src, B.pos1, B.vel1, B.aux[cur], B.start,
-                     ain, vpd, out, dbg_for(t), P.counters, B.err);
+        if (by_warp && mode == MODE_RECORD)
+            warp_solve_kernel<SRC, MODE_RECORD><<<wgrid, sb, 0, st>>>(
+                n, src, B.pos1, B.vel1, B.aux[cur], B.start, ain, vpd, out, dbg_for(t), B.err);
+        else if (by_warp)
+            warp_solve_kernel<SRC, MODE_PLAIN><<<wgrid, sb, 0, st>>>(
+                n, src, B.pos1, B.vel1, B.aux[cur], B.start, ain, vpd, out, dbg_for(t), B.err);
+        else
+            launch_solve(mode, sgrid, sb, smem, st, n, src, B.pos1, B.vel1, B.aux[cur], B.start,
+                         ain, vpd, out, dbg_for(t), P.counters, B.err);
         if (P.ev_end) cudaEventRecord(P.ev_end, st);
         nvtxRangePop();
     }
