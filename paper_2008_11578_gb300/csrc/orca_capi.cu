@@ -24,6 +24,7 @@
 
 #include "orca.h"
 #include "orca_adjoint.cuh"
+#include "orca_cluster_bin.cuh"
 #include "orca_step_kernels.cuh"
 #include "orca_warp_solve.cuh"
 
@@ -263,6 +264,33 @@ void launch_solve(int mode, int grid, int block, size_t smem, cudaStream_t st, i
 #undef ORCA_SOLVE
 }
 
+// The kernel may be set up while the one before it in the stream still runs
+// (it waits for that one's end itself, see wait_for_primary).
+cudaLaunchAttribute programmatic_launch() {
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    return a;
+}
+
+template <class SRC>
+void launch_warp_solve(int mode, int grid, int block, cudaStream_t st, int n, SRC src,
+                       const float2* pos, const float2* vel, const uint2* aux,
+                       const uint32_t* start, AgentIn ain, const float2* vpd, StepOut out,
+                       DebugOut dbg, int* err) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1] = {programmatic_launch()};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg,
+                       mode == MODE_RECORD ? warp_solve_kernel<SRC, MODE_RECORD>
+                                           : warp_solve_kernel<SRC, MODE_PLAIN>,
+                       n, src, pos, vel, aux, start, ain, vpd, out, dbg, err);
+}
+
 // Everything one call of the step pipeline needs: the caller's arrays, the
 // workspace and the launch shape.  n_scenes == 0 is a single scene (its
 // constants passed by value), otherwise a batch.
@@ -287,6 +315,7 @@ struct Pipeline {
     cudaGraphExec_t graph;
     int graph_steps;
     int bin_grid_max;   // co-resident blocks of the binning kernel on this device
+    int cluster_max;    // blocks of the largest cluster that runs here (small scenes)
 };
 
 size_t solve_smem(const Pipeline& P) { return (size_t)P.kcap * P.block * sizeof(float4); }
@@ -319,10 +348,36 @@ bool solve_by_warp(const Pipeline& P, int mode) {
            P.n <= (P.kcap <= 16 ? kWarpSolveMax : kWarpSolveMaxWide);
 }
 
+// Largest scene binned by a cluster.  Against bin_kernel (first step of a call
+// / later steps): 1,000 agents 18 / 14 us -> 14 / 10 us, 16,000 agents
+// 22 / 16 -> 15 / 12 us, 32,000 agents 23 / 16 -> 20 / 14 us; a scene's very
+// first step, in the caller's order, 26 -> 16 us at 1,000, 25 -> 23 us at 16,000
+// and 26 -> 32 us at 32,000, where the 16 SMs of the cluster fall behind.
+constexpr int kClusterBinMax = 20480;
+static_assert(kClusterBinMax <= kClusterMax * kClusterSlots, "a cluster holds the scene");
+
+// Blocks of the cluster that bins the scene (0: it takes bin_kernel instead):
+// about one agent per thread, more where the cells need the shared memory.
+int bin_cluster(const Pipeline& P, ClusterShape* sh) {
+    if (P.n > kClusterBinMax || (P.flags & ORCA_DEBUG_BARRIER_TIMEOUT)) return 0;
+    for (int nb = 1; nb <= P.cluster_max; nb *= 2) {
+        const bool last = nb * 2 > P.cluster_max;
+        ClusterShape s{2, 0};
+        while (((long long)nb << s.cell_shift) < P.ncells) ++s.cell_shift;
+        while (((long long)nb << s.slot_shift) < P.n) ++s.slot_shift;
+        if ((1 << s.cell_shift) > kClusterCells) continue;
+        if ((1 << s.slot_shift) > (last ? kClusterSlots : kClusterThreads)) continue;
+        *sh = s;
+        return nb;
+    }
+    return 0;
+}
+
 // The binning kernel of one step (cooperative launch, grid sized to what is
 // resident at once on this device).  first: from the caller's arrays.
 template <class SRC>
-void launch_bin(const Pipeline& P, SRC src, bool first, int cur, cudaStream_t st) {
+void launch_bin(const Pipeline& P, SRC src, bool first, int cur, int nb, ClusterShape sh,
+                cudaStream_t st) {
     const Buffers& B = P.buf;
     const orca_agents& A = P.agents;
     const BinArgs a{P.n, P.ncells, (const float2*)A.pos, (const float2*)A.vel, A.radius, A.type,
@@ -330,6 +385,23 @@ void launch_bin(const Pipeline& P, SRC src, bool first, int cur, cudaStream_t st
                     B.count, B.start, B.bsum, B.xrank,
                     B.pos1, B.vel1, B.aux[1 - cur], B.err, B.hint,
                     (P.flags & ORCA_DEBUG_BARRIER_TIMEOUT) ? 1 : 0};
+    if (nb > 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)nb);
+        cfg.blockDim = dim3(kClusterThreads);
+        cfg.dynamicSmemBytes = cluster_smem(sh);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)nb;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        attr[1] = programmatic_launch();
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        if (first) cudaLaunchKernelEx(&cfg, cluster_bin_kernel<SRC, true>, src, a, sh);
+        else cudaLaunchKernelEx(&cfg, cluster_bin_kernel<SRC, false>, src, a, sh);
+        return;
+    }
     const long long work = std::max((long long)P.n, (long long)P.ncells / 4);
     const int grid = (int)std::max(
         1LL, std::min((long long)P.bin_grid_max, (work + kBinThreads - 1) / kBinThreads));
@@ -362,6 +434,8 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
     const int sgrid = (n + sb - 1) / sb;
     const size_t smem = solve_smem(P);
     const bool by_warp = solve_by_warp(P, mode);
+    ClusterShape shape{0, 0};
+    const int nb = bin_cluster(P, &shape);
     const int wgrid = (int)(((long long)n * 32 + sb - 1) / sb);
     // NVTX ranges (host side: the enqueue of each step and its two kernels)
     nvtxRangePushA("orca_step");
@@ -370,7 +444,7 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
         if (P.bin_begin) cudaEventRecord(P.bin_begin, st);
         // step 0 bins the caller's state; later steps were binned by the
         // previous step's solve kernel
-        launch_bin(P, src, t == 0, cur, st);
+        launch_bin(P, src, t == 0, cur, nb, shape, st);
         cur = 1 - cur;
         if (P.bin_end) cudaEventRecord(P.bin_end, st);
         nvtxRangePop();
@@ -381,14 +455,11 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
         const bool last = t == n_steps - 1;
         const StepOut out = last ? StepOut{(float2*)A.pos, (float2*)A.vel, true, nullptr, nullptr,
                                            nullptr, B.hint, B.err + 1}
-                                 : StepOut{B.pos0, B.vel0, false, B.key, B.slot, B.count,
-                                           nullptr, nullptr};
-        if (by_warp && mode == MODE_RECORD)
-            warp_solve_kernel<SRC, MODE_RECORD><<<wgrid, sb, 0, st>>>(
-                n, src, B.pos1, B.vel1, B.aux[cur], B.start, ain, vpd, out, dbg_for(t), B.err);
-        else if (by_warp)
-            warp_solve_kernel<SRC, MODE_PLAIN><<<wgrid, sb, 0, st>>>(
-                n, src, B.pos1, B.vel1, B.aux[cur], B.start, ain, vpd, out, dbg_for(t), B.err);
+                                 : StepOut{B.pos0, B.vel0, false, nb > 0 ? nullptr : B.key,
+                                           B.slot, B.count, nullptr, nullptr};
+        if (by_warp)
+            launch_warp_solve(mode, wgrid, sb, st, n, src, B.pos1, B.vel1, B.aux[cur], B.start,
+                              ain, vpd, out, dbg_for(t), B.err);
         else
             launch_solve(mode, sgrid, sb, smem, st, n, src, B.pos1, B.vel1, B.aux[cur], B.start,
                          ain, vpd, out, dbg_for(t), P.counters, B.err);
@@ -424,6 +495,44 @@ cudaError_t bin_grid_max(int* out) {
     return e;
 }
 
+// Blocks of the largest cluster of the small-scene binning kernel that the
+// current device runs (0: none).
+template <class SRC>
+cudaError_t cluster_max(int* out) {
+    *out = 0;
+    const size_t smem = (size_t)16 * kClusterSlots + (size_t)4 * kClusterCells + 16;
+    for (auto f : {cluster_bin_kernel<SRC, true>, cluster_bin_kernel<SRC, false>}) {
+        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+    }
+    for (int nb = kClusterMax; nb >= 1; nb /= 2) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)nb);
+        cfg.blockDim = dim3(kClusterThreads);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)nb;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int k0 = 0, k1 = 0;
+        if (cudaOccupancyMaxActiveClusters(&k0, cluster_bin_kernel<SRC, true>, &cfg) ==
+                cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&k1, cluster_bin_kernel<SRC, false>, &cfg) ==
+                cudaSuccess &&
+            k0 > 0 && k1 > 0) {
+            *out = nb;
+            break;
+        }
+    }
+    cudaGetLastError();   // a size that does not fit is no error of the caller's
+    return cudaSuccess;
+}
+
 int prepare(Pipeline& P) {
     const size_t smem = solve_smem(P);
     cudaError_t e = P.n_scenes == 0 ? prepare_solve<OneScene>(smem)
@@ -431,6 +540,9 @@ int prepare(Pipeline& P) {
     if (e == cudaSuccess)
         e = P.n_scenes == 0 ? bin_grid_max<OneScene>(&P.bin_grid_max)
                             : bin_grid_max<ManyScenes>(&P.bin_grid_max);
+    if (e == cudaSuccess)
+        e = P.n_scenes == 0 ? cluster_max<OneScene>(&P.cluster_max)
+                            : cluster_max<ManyScenes>(&P.cluster_max);
     return cuda_status(e);
 }
 
@@ -530,6 +642,7 @@ void init_pipeline(Pipeline& P, const orca_agents* agents, int ncells, int kcap,
     P.graph = nullptr;
     P.graph_steps = 0;
     P.bin_grid_max = 1;
+    P.cluster_max = 0;
 }
 
 // Host-side checks of a batch description; fills the total cell count and

@@ -1,0 +1,185 @@
+// orca_cluster_bin.cuh -- the binning step of small scenes as one
+// thread-block cluster (sm_103a).
+//
+// bin_kernel sorts the agents through global memory in phases separated by
+// grid barriers; with few agents each phase is a few dependent L2 round trips
+// and a barrier, 16 us a step however small the scene.  Here the cell counts,
+// the cell starts and the cell-order records live in the shared memory of at
+// most 16 blocks of one cluster: block r owns a contiguous range of cells and
+// a contiguous range of slots, the others reach them through distributed
+// shared memory, and the hardware cluster barrier (every block of a cluster is
+// resident) separates the phases.  The sorted state is the same as
+// bin_kernel's up to the order of agents with equal cell and x, which no
+// result depends on.
+#pragma once
+
+#include <cooperative_groups.h>
+
+#include "orca_step_kernels.cuh"
+
+namespace orca {
+
+constexpr int kClusterMax = 16;
+constexpr int kClusterThreads = 1024;
+constexpr int kClusterPerThread = 2;                                 // agents
+constexpr int kClusterSlots = kClusterThreads * kClusterPerThread;   // per block
+constexpr int kClusterCells = 32768;                                 // per block
+
+// log2 sizes of the cell and slot ranges of a block
+struct ClusterShape {
+    int cell_shift;
+    int slot_shift;
+};
+
+inline size_t cluster_smem(ClusterShape sh) {
+    return ((size_t)16 << sh.slot_shift) + ((size_t)4 << sh.cell_shift) + 16;
+}
+
+template <class SRC, bool FIRST>
+__global__ void __launch_bounds__(kClusterThreads)
+cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
+    namespace cg = cooperative_groups;
+    extern __shared__ uint4 cluster_mem[];
+    __shared__ uint32_t ws[32], total, base[kClusterMax + 1];
+    const cg::cluster_group cl = cg::this_cluster();
+    const int r = (int)blockIdx.x, nb = (int)gridDim.x, tid = (int)threadIdx.x;
+    const int cn = 1 << sh.cell_shift, sn = 1 << sh.slot_shift;
+    uint4* slots = cluster_mem;                                    // sn cell-order records
+    uint32_t* cells = reinterpret_cast<uint32_t*>(slots + sn);     // cn counts, then starts, + total
+
+    // the solve kernel may be set up meanwhile; what ran before is finished
+    // before any state is read
+    launch_dependents();
+    wait_for_primary();
+
+    // ---- the agents of this block and their cells ----
+    // (first step: in the order that the previous call recorded, if it did, so
+    // that a block's agents lie in few blocks' cells)
+    const uint32_t* __restrict__ hint = nullptr;
+    if (FIRST && __ldcg(a.err + 1) != 0) hint = a.hint;
+    const int i0 = r << sh.slot_shift;
+    const int iend = min(i0 + sn, a.n);
+    int from[kClusterPerThread];
+    float x[kClusterPerThread];
+    uint32_t c[kClusterPerThread];
+    bool bad = false, lost = false;
+#pragma unroll
+    for (int u = 0; u < kClusterPerThread; ++u) {
+        from[u] = i0 + tid + u * kClusterThreads;
+        if (FIRST && hint != nullptr && from[u] < iend) {
+            const uint32_t h = __ldg(hint + from[u]);
+            if (h < (uint32_t)a.n) from[u] = (int)h;
+            else lost = true;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kClusterPerThread; ++u) {
+        c[u] = 0xffffffffu;
+        x[u] = 0.0f;
+        if (i0 + tid + u * kClusterThreads < iend) {
+            const int i = from[u];
+            const float2 p = FIRST ? a.upos[i] : a.pos0[i];
+            if (FIRST) {
+                const float2 v = a.uvel[i];
+                bad |= !(isfinite(p.x) && isfinite(p.y) && isfinite(v.x) && isfinite(v.y));
+            }
+            const SceneDev& sc = src.get(i);
+            x[u] = p.x;
+            c[u] = (uint32_t)(sc.cell_off +
+                              cell_axis(p.y, sc.origin_y, sc.inv_cell_y, sc.ny) * sc.nx +
+                              cell_axis(p.x, sc.origin_x, sc.inv_cell_x, sc.nx));
+        }
+    }
+    if (lost) atomicOr(a.err, ERR_BIT_STATE);
+    for (int q = tid; q <= cn; q += kClusterThreads) cells[q] = 0u;
+    if (bad) atomicOr(a.err, ERR_BIT_NONFINITE);
+    cl.sync();
+
+    // ---- counting ----
+    uint32_t slot[kClusterPerThread];
+#pragma unroll
+    for (int u = 0; u < kClusterPerThread; ++u) {
+        slot[u] = 0u;
+        if (c[u] != 0xffffffffu) {
+            uint32_t* rc = cl.map_shared_rank(cells, (unsigned)(c[u] >> sh.cell_shift));
+            slot[u] = atomicAdd(rc + (c[u] & (uint32_t)(cn - 1)), 1u);
+        }
+    }
+    cl.sync();
+
+    // ---- starts within the block's cells, and the blocks' totals ----
+    {
+        uint32_t carry = 0u;
+        for (int q0 = 0; q0 < cn; q0 += 4 * kClusterThreads) {
+            const int q = q0 + 4 * tid;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (q < cn) v = *reinterpret_cast<const uint4*>(cells + q);
+            uint32_t tile;
+            const uint32_t o = carry + block_excl_scan(v.x + v.y + v.z + v.w, ws, tile);
+            if (q < cn)
+                *reinterpret_cast<uint4*>(cells + q) =
+                    make_uint4(o, o + v.x, o + v.x + v.y, o + v.x + v.y + v.z);
+            carry += tile;
+        }
+        if (tid == 0) {
+            cells[cn] = carry;
+            total = carry;
+        }
+    }
+    cl.sync();
+    if (tid < 32) {
+        uint32_t t = tid < nb ? *cl.map_shared_rank(&total, (unsigned)tid) : 0u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
+            if (tid >= o) t += y;
+        }
+        if (tid < nb) base[tid + 1] = t;
+        if (tid == 0) base[0] = 0u;
+    }
+    __syncthreads();
+
+    // ---- records into cell order; the starts for the search ----
+#pragma unroll
+    for (int u = 0; u < kClusterPerThread; ++u) {
+        if (c[u] != 0xffffffffu) {
+            const unsigned own = (unsigned)(c[u] >> sh.cell_shift);
+            const uint32_t* rc = cl.map_shared_rank(cells, own) + (c[u] & (uint32_t)(cn - 1));
+            const uint32_t b = base[own] + rc[0], e = base[own] + rc[1], d = b + slot[u];
+            uint4* rs = cl.map_shared_rank(slots, (unsigned)(d >> sh.slot_shift));
+            rs[d & (uint32_t)(sn - 1)] = make_uint4(x_order_key(x[u]), (uint32_t)from[u], b, e);
+        }
+    }
+    const int c0 = r << sh.cell_shift;
+    for (int q = tid; q < cn && c0 + q < a.ncells; q += kClusterThreads)
+        a.start[c0 + q] = base[r] + cells[q];
+    if (r == nb - 1 && tid == 0) a.start[a.ncells] = (uint32_t)a.n;
+    cl.sync();
+
+    // ---- order by x inside every cell (ties by slot); move the state ----
+#pragma unroll
+    for (int u = 0; u < kClusterPerThread; ++u) {
+        const int t = i0 + tid + u * kClusterThreads;
+        if (t < iend) {
+            const uint4 e = slots[t - i0];
+            const uint32_t i = e.y;
+            const float2 p = FIRST ? a.upos[i] : a.pos0[i];
+            const float2 v = FIRST ? a.uvel[i] : a.vel0[i];
+            const uint2 ax = FIRST ? aux_pack(a.urad[i], a.utype[i], (int)i) : a.aux0[i];
+            uint32_t rank = 0u;
+            for (uint32_t w = e.z; w < e.w; ++w) {
+                const unsigned own = (unsigned)(w >> sh.slot_shift);
+                const uint4* rs = own == (unsigned)r ? slots : cl.map_shared_rank(slots, own);
+                const uint32_t xv = rs[w & (uint32_t)(sn - 1)].x;
+                rank += (xv < e.x || (xv == e.x && w < (uint32_t)t)) ? 1u : 0u;
+            }
+            const uint32_t dst = e.z + rank;
+            a.pos1[dst] = p;
+            a.vel1[dst] = v;
+            a.aux1[dst] = ax;
+        }
+    }
+    cl.sync();   // no block leaves while another reads its records
+}
+
+}  // namespace orca

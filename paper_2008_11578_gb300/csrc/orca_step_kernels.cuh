@@ -10,6 +10,19 @@
 
 namespace orca {
 
+// ------------------------------------------------- programmatic launches ----
+// Kernels launched with programmatic stream serialisation start while the
+// kernel before them still runs, once all its blocks have called
+// launch_dependents() (or exited); wait_for_primary() returns when that
+// kernel has finished and its writes are visible.  Without the launch
+// attribute both do nothing.
+__device__ __forceinline__ void launch_dependents() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_primary() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ------------------------------------------------------------------ scan ----
 // Exclusive scan of the cell counts into cell starts, three phases: per-block
 // scan of kScanChunk cells (writing block totals), scan of the block totals

@@ -237,6 +237,8 @@ warp_solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* 
     const int lane = threadIdx.x & 31;
     WarpSlots& W = slots[threadIdx.x >> 5];
     const int s = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    launch_dependents();
+    wait_for_primary();
     if (s >= n) return;
     const SceneDev& sc = src.get(s);
     const int status = __ldcg(err);
