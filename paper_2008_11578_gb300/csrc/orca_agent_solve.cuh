@@ -1,0 +1,487 @@
+// orca_agent_solve.cuh -- the solve kernel with one thread per agent (sm_103a).
+//
+// Search: the k + 1 smallest distances are kept sorted in registers by a
+// network of minima and maxima (no branches: the 32 lanes of a warp insert
+// whatever their candidates are).  An entry is the distance d^2 with its lowest
+// bits replaced by the candidate's place in a list of admitted slots in shared
+// memory, so the order of the neighbours falls out of the network.  Where two
+// distances differ only in the replaced bits (some 5e-4 of the agents, or
+// lattices) the list is put in order exactly.
+//
+// Bound by issue slots (0.71 of one instruction a cycle per scheduler, 44 % of
+// an instruction's lanes active: the LP's re-solves and the half-planes'
+// constructions differ between the lanes) in large scenes, by one thread's chain
+// in smaller ones.  1M clusters, first step of a call: 454 us with the sorted
+// list in shared memory, 420 with the network and a pass that ranks the admitted
+// slots, 394 with the places carried in the entries, 377-380 with the LP's order
+// by all pairs and the penetrations kept for the LP (65,000-agent shared space:
+// 67, 55, 58, 52).  Of it the row scan takes about 90 us, the network 60, the
+// half-planes 58, the LP 130.  Seven blocks an SM (72 registers) measured 380 us
+// there and 73 us at 130,000 agents, six 403 and 88, eight 377 and 76, nine 396
+// and 79.
+#pragma once
+
+#include "orca_step_kernels.cuh"
+
+namespace orca {
+
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// The N smallest of the sorted D and of a and b.  The i-th smallest of the
+// union is min(D[i], max(D[i - 1], x), max(D[i - 2], y)) for x <= y.
+template <int N>
+__device__ __forceinline__ void insert_pair(float (&D)[N], float a, float b) {
+    const float x = fminf(a, b), y = fmaxf(a, b);
+#pragma unroll
+    for (int i = N - 1; i >= 2; --i) D[i] = min3(D[i], fmaxf(D[i - 1], x), fmaxf(D[i - 2], y));
+    D[1] = min3(D[1], fmaxf(D[0], x), y);
+    D[0] = fminf(D[0], x);
+}
+
+// Shared memory of a warp, in 16-byte units per lane: kl line slots, then kl
+// words (the neighbours in order, then each line's penetration at v_A).  The
+// search's list of admitted slots lives in the line slots.
+__host__ __device__ constexpr int agent_units(int kl) { return kl + (kl + 3) / 4; }
+
+// One thread per agent (sorted slot s), k <= KC, the incremental LP.
+// MODE_PLAIN, or MODE_RECORD with the LP's active set.  kl: line slots per
+// lane (KC, and the kinematic half-planes if the scene has them).
+template <class SRC, int MODE, int KC>
+__global__ void __launch_bounds__(128, KC <= 10 ? 7 : 1)
+agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
+                   const float2* __restrict__ vel, const uint2* __restrict__ aux,
+                   const uint32_t* __restrict__ cstart, AgentIn ain,
+                   const float2* __restrict__ vpd, StepOut out, DebugOut dbg,
+                   int* __restrict__ err) {
+    extern __shared__ float4 smem_lines[];
+    // after a binning kernel that gave up or found inconsistent counts the
+    // sorted state is not valid: leave everything as it is (the status call
+    // reports the error)
+    if (__ldcg(err) & (ERR_BIT_TIMEOUT | ERR_BIT_STATE)) return;
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned lanes = __ballot_sync(0xffffffffu, s < n);
+    if (s >= n) return;
+    float4* L = smem_lines + (threadIdx.x >> 5) * agent_units(kl) * 32 + (threadIdx.x & 31);
+    int* J = reinterpret_cast<int*>(L - (threadIdx.x & 31) + kl * 32) + (threadIdx.x & 31);
+    int* raw = reinterpret_cast<int*>(L - (threadIdx.x & 31)) + (threadIdx.x & 31);
+    // low bits of an entry of the network: a place in raw
+    constexpr uint32_t kPlace = KC <= 16 ? 63u : 127u;
+    const int cap = min(4 * kl, (int)kPlace);   // entries of raw
+    const SceneDev& sc = src.get(s);
+    const float2 p = pos[s];
+    const float2 v = vel[s];
+    const uint2 as = aux[s];
+    const float r = aux_rad(as);
+    const int ta = aux_type(as);
+    const int o = aux_orig(as);
+    const int cx = cell_axis(p.x, sc.origin_x, sc.inv_cell_x, sc.nx);
+    const int cy = cell_axis(p.y, sc.origin_y, sc.inv_cell_y, sc.ny);
+
+    // ---- k nearest by (d^2, index), exact search over the x-sorted grid rows ----
+    const int k = sc.k;
+    int cnt = 0;
+    if (k > 0 && isfinite(p.x) && isfinite(p.y)) {   // (a non-finite state is an error)
+        const float R2 = sc.R2;
+        // the largest float below R_n^2: a candidate within the bound (this, or
+        // the k-th distance once k are known, its low bits set) is admitted,
+        // and a row cursor stops beyond it
+        const float thr0 = R2 > 0.0f ? __int_as_float(__float_as_int(R2) - 1) : -1.0f;
+        // sorted; the first KC - k entries are below every distance, the ones
+        // not yet found above
+        float D[KC + 1];
+        auto clear = [&]() {
+#pragma unroll
+            for (int i = 0; i <= KC; ++i)
+                D[i] = i < KC - k ? -1.0f : __uint_as_float(__float_as_uint(thr0) | kPlace);
+        };
+        auto bound = [&]() {
+            return fminf(thr0, __uint_as_float(__float_as_uint(D[KC - 1]) | kPlace));
+        };
+        auto entry = [](float d2, int place) {
+            return __uint_as_float((__float_as_uint(d2) & ~kPlace) | (uint32_t)place);
+        };
+        clear();
+        const uint32_t* __restrict__ cs = cstart + sc.cell_off;
+        const uint32_t* __restrict__ aux_idx = reinterpret_cast<const uint32_t*>(aux) + 1;
+        int found = 0;
+        // whether list entry e comes before candidate (d2, oj)
+        auto before = [&](int e, float d2, int oj) {
+            const int j = raw[e * 32];
+            const float2 q = pos[j];
+            const float de = key_d2(p.x, p.y, q.x, q.y);
+            return de < d2 ||
+                   (de == d2 && aux_orig(make_uint2(0u, __ldg(aux_idx + 2 * j))) < oj);
+        };
+        // make room: keep the entries within the bound; should that not be
+        // enough (many equal distances), the k first by (d^2, index)
+        auto compact = [&](float lim, int room) {
+            int kept = 0;
+            for (int e = 0; e < found; ++e) {
+                const int j = raw[e * 32];
+                const float2 q = pos[j];
+                if (key_d2(p.x, p.y, q.x, q.y) <= lim) raw[32 * kept++] = j;
+            }
+            found = kept;
+            while (found > room && found > k) {   // drop the last by (d^2, index)
+                int last = 0;
+                for (int e = 1; e < found; ++e) {
+                    const int j = raw[e * 32];
+                    const float2 q = pos[j];
+                    if (before(last, key_d2(p.x, p.y, q.x, q.y),
+                               aux_orig(make_uint2(0u, __ldg(aux_idx + 2 * j)))))
+                        last = e;
+                }
+                --found;
+                raw[last * 32] = raw[found * 32];
+            }
+        };
+        // Every grid row is one run of slots sorted by x (the binning kernel
+        // orders each cell by x, and cells of a row are consecutive in x).
+        // A row is scanned outward from the agent's x with two cursors: the
+        // right one stops at the first candidate right of the agent whose
+        // fl(dx^2 + g2) exceeds the bound, the left one likewise on the left,
+        // where g2 is the row's lower bound of dy^2; every candidate farther
+        // along has a larger dx^2, and d^2 = fl(dx^2 + dy^2) >= fl(dx^2 + g2)
+        // (rounding is monotone), so none of them can enter the list.
+        // Any start slot is valid (candidates on the wrong side of the agent
+        // never stop a cursor); a good start only saves candidate tests.
+        // Rows are visited nearest first (the agent's own row, then one row
+        // on each side in turn, the nearer of the two first) and a side ends
+        // at the first row whose y gap is beyond the bound.
+        const int nx = sc.nx, ny = sc.ny;
+        const float ch = sc.cell_h, mg = sc.ring_delta * ch;
+        const float pry = __fsub_rn(p.y, sc.origin_y);
+        // lower bound of dy^2 for every agent binned into row ry (widened by
+        // the cell-rounding margin, open toward the grid edge), with the
+        // 1e-5 relative slack of the key comparison
+        auto row_gap2 = [&](int ry) {
+            const float by0 = ry == 0 ? -CUDART_INF_F : (float)ry * ch - mg;
+            const float by1 = ry == ny - 1 ? CUDART_INF_F : (float)(ry + 1) * ch + mg;
+            const float ey = fmaxf(fmaxf(by0 - pry, pry - by1), 0.0f);
+            return ey * ey * 0.99999f;
+        };
+        // start slot of row ry: the agent's x interpolated inside the row's
+        // cell of column cx (x-sorted, so agents spread roughly evenly)
+        const float fx = fminf(fmaxf(__fmul_rn(__fsub_rn(p.x, sc.origin_x), sc.inv_cell_x) -
+                                         (float)cx, 0.0f), 1.0f);
+        // Rows in visiting order, through one copy of the row scan: the agent's
+        // own row (ring 0) from its neighbouring slots (the agent itself is
+        // never a candidate), then ring by ring the nearer of rows cy - m and
+        // cy + m first.
+        bool up = true, down = true;   // rows cy + m / cy - m left to visit
+        int m = 0, so = 2;             // ring, and the next of its two sides
+        float gd = 0.0f, gu = 0.0f;    // the ring's y gaps below and above
+        int first = 0;
+        int ry = cy, jr = s + 1, jl = s - 1;
+        float g2 = 0.0f;
+        for (;;) {
+            const int rb = (int)__ldg(cs + ry * nx), re = (int)__ldg(cs + ry * nx + nx);
+            bool ron = jr < re, lon = jl >= rb;
+            float2 nr = pos[min(jr, n - 1)], nl = pos[max(jl, 0)];
+            while (ron || lon) {
+                // the next candidates are on their way while these are tested
+                const float2 qr = nr, ql = nl;
+                nr = pos[min(jr + 1, n - 1)], nl = pos[max(jl - 1, 0)];
+                const float lim = bound();
+                const float dxr = __fsub_rn(qr.x, p.x), dxl = __fsub_rn(ql.x, p.x);
+                const float xxr = __fmul_rn(dxr, dxr), xxl = __fmul_rn(dxl, dxl);
+                ron = ron && !(dxr > 0.0f && __fadd_rn(xxr, g2) > lim);
+                lon = lon && !(dxl < 0.0f && __fadd_rn(xxl, g2) > lim);
+                const float dyr = __fsub_rn(qr.y, p.y), dyl = __fsub_rn(ql.y, p.y);
+                float dr = __fadd_rn(xxr, __fmul_rn(dyr, dyr));
+                float dl = __fadd_rn(xxl, __fmul_rn(dyl, dyl));
+                if (!ron || dr > lim) dr = CUDART_INF_F;
+                if (!lon || dl > lim) dl = CUDART_INF_F;
+                float er = dr, el = dl;
+                if (dr < CUDART_INF_F) {
+                    er = entry(dr, found);
+                    raw[found++ * 32] = jr;
+                }
+                if (dl < CUDART_INF_F) {
+                    el = entry(dl, found);
+                    raw[found++ * 32] = jl;
+                }
+                insert_pair<KC + 1>(D, er, el);
+                ron = ron && ++jr < re;
+                lon = lon && --jl >= rb;
+                if (found > cap - 2) {
+                    compact(bound(), cap / 2);
+                    clear();
+                    for (int e = 0; e < found; ++e) {
+                        const float2 q = pos[raw[e * 32]];
+                        insert_pair<KC + 1>(D, entry(key_d2(p.x, p.y, q.x, q.y), e),
+                                            CUDART_INF_F);
+                    }
+                }
+            }
+            bool more = false;
+            while (!more && (up || down)) {
+                if (so == 2) {
+                    ++m;
+                    so = 0;
+                    gd = row_gap2(cy - m);
+                    gu = row_gap2(cy + m);
+                    first = gu < gd ? 1 : 0;
+                }
+                const int side = so ^ first;
+                ++so;
+                if (!(side == 0 ? down : up)) continue;
+                ry = side == 0 ? cy - m : cy + m;
+                g2 = side == 0 ? gd : gu;
+                if (ry < 0 || ry >= ny || g2 > bound()) {
+                    if (side == 0) down = false;
+                    else up = false;
+                    continue;
+                }
+                more = true;
+            }
+            if (!more) break;
+            const int c = ry * nx + cx;
+            const int b = (int)__ldg(cs + c), e = (int)__ldg(cs + c + 1);
+            jr = min(b + (int)(fx * (float)(e - b)), e);
+            jl = jr - 1;
+        }
+        cnt = min(found, k);
+        // the neighbours in order: entry KC - k + m is the m-th, unless entries
+        // that follow one another differ in the replaced bits only
+        const int fill = KC - k;
+        bool tie = false;
+#pragma unroll
+        for (int i = 0; i < KC; ++i) {
+            const uint32_t a = __float_as_uint(D[i]), b = __float_as_uint(D[i + 1]);
+            const int at = i - fill;
+            if (at >= 0 && at < cnt) {
+                J[at * 32] = raw[(int)(a & kPlace) * 32];
+                tie |= (a ^ b) <= kPlace && at + 1 < found;
+            }
+        }
+        if (tie) {   // the k first by (d^2, index), in that order
+            compact(bound(), cap);
+            for (int e = 0; e < found; ++e) {
+                const int j = raw[e * 32];
+                const float2 q = pos[j];
+                const float d2 = key_d2(p.x, p.y, q.x, q.y);
+                const int oj = aux_orig(make_uint2(0u, __ldg(aux_idx + 2 * j)));
+                int at = 0;
+                for (int u = 0; u < found; ++u) at += u != e && before(u, d2, oj) ? 1 : 0;
+                if (at < k) J[at * 32] = j;
+            }
+        }
+    }
+    __syncwarp(lanes);   // the lines take the place of the lists
+
+    // ---- preferred velocity toward the goal or the current waypoint ----
+    float2 g = ain.goal[o];
+    const float vmax = ain.max_speed[o];
+    if (ain.route != nullptr) {
+        const int rt = ain.route[o];
+        if (rt >= 0) {
+            int wi = ain.wp_idx[o];
+            if (dbg.swp != nullptr) dbg.swp[o] = (uint8_t)wi;
+            wi = advance_waypoint(ain.waypoints + (size_t)rt * ain.n_waypoints, ain.n_waypoints,
+                                  wi, p, r, g);
+            ain.wp_idx[o] = (uint8_t)wi;
+            if (dbg.wp_used != nullptr) dbg.wp_used[o] = (uint8_t)wi;
+        }
+    }
+    const float2 vp = preferred_velocity(p, g, vmax, sc.inv_dt, vpd != nullptr,
+                                         vpd != nullptr ? vpd[o] : make_float2(0.0f, 0.0f));
+
+    // ---- one ORCA half-plane per neighbour (Sec. 3.1) ----
+    // Constraint m is the m-th nearest.  pen[m], its penetration at v_A, takes
+    // the place of the neighbour's slot.
+    if (dbg.nbr != nullptr) {
+        int32_t* nb = dbg.nbr + (size_t)o * dbg.k_stride;
+        for (int m = 0; m < dbg.k_stride; ++m)
+            nb[m] = m < cnt ? aux_orig(aux[J[m * 32]]) : -1;
+    }
+    float* pen = reinterpret_cast<float*>(J);
+    bool any_overlap = false;
+    uint32_t capbits = 0u, ovbits = 0u;   // per-line construction (MODE_RECORD)
+    int nlines = 0;
+    // the two lines most violated at v_A so far
+    float pm0 = -CUDART_INF_F, pm1 = -CUDART_INF_F;
+    int im0 = -1, im1 = -1;
+    auto add_line = [&](float4 l) {
+        const float pv = penetration(l, v.x, v.y);
+        L[nlines * 32] = l;
+        pen[nlines * 32] = pv;
+        if (pv > pm0) {
+            pm1 = pm0;
+            im1 = im0;
+            pm0 = pv;
+            im0 = nlines;
+        } else if (pv > pm1) {
+            pm1 = pv;
+            im1 = nlines;
+        }
+        ++nlines;
+    };
+    for (int i = 0; i < cnt; ++i) {
+        const int j = J[i * 32];
+        const float2 pj = pos[j], vj = vel[j];
+        const uint2 aj = aux[j];
+        const float rj = aux_rad(aj);
+        const int tb = aux_type(aj);
+        const float rs = __fadd_rn(r, rj);
+        const bool ov = key_d2(p.x, p.y, pj.x, pj.y) <= __fmul_rn(rs, rs);
+        any_overlap |= ov;
+        const float f = tb ? (ta ? sc.f11 : sc.f01) : (ta ? sc.f10 : sc.f00);
+        bool cap_line;
+        add_line(orca_line(p.x, p.y, v.x, v.y, r, pj.x, pj.y, vj.x, vj.y, rj, f, sc.inv_tau,
+                           sc.inv_dt, ov, cap_line));
+        if (MODE == MODE_RECORD) {
+            ovbits |= (ov ? 1u : 0u) << i;
+            capbits |= (cap_line ? 1u : 0u) << i;
+        }
+    }
+
+    // ---- vehicles' kinematic half-planes (off unless the scene sets limits) ----
+    if (ta != 0 && (sc.kin_turn || sc.kin_accel)) limit_lines(sc, v, vp, add_line);
+
+    // ---- constraint order of the LP ----
+    // Half-planes in decreasing penetration at the agent's current velocity:
+    // the least-penetration optimum usually rests on the most violated ones,
+    // so fewer of the later lines force a re-solve.  The two most violated
+    // go first (swaps: slot 0 <-> sw0, then slot 1 <-> sw1); with at most 16
+    // lines the rest follow in sorted order (ties keep their order).  The LP's
+    // result does not depend on the order beyond rounding; the recorded
+    // active set is mapped back to the neighbour order below, through perm
+    // (slot -> neighbour index, 4 bits per slot) when sorted.
+    int sw0 = 0, sw1 = 1;
+    auto swap_lines = [&](int a, int b) {
+        const float4 l = L[a * 32];
+        const float q = pen[a * 32];
+        L[a * 32] = L[b * 32];
+        pen[a * 32] = pen[b * 32];
+        L[b * 32] = l;
+        pen[b * 32] = q;
+    };
+    if (nlines > 1) {
+        if (im0 > 0) {
+            swap_lines(0, im0);
+            sw0 = im0;
+        }
+        if (im1 >= 0 && nlines > 2) {
+            const int b = im1 == 0 ? sw0 : im1;   // where the second line is now (>= 1)
+            if (b > 1) {
+                swap_lines(1, b);
+                sw1 = b;
+            }
+        }
+    }
+    auto nib = [](uint64_t q, int i) { return (uint32_t)((q >> (4 * i)) & 15ull); };
+    auto put = [](uint64_t q, int i, uint32_t x) {
+        return (q & ~(15ull << (4 * i))) | ((uint64_t)x << (4 * i));
+    };
+    uint64_t perm = 0ull;
+    if (MODE == MODE_RECORD && nlines <= 16) {
+        perm = 0xFEDCBA9876543210ull;
+        const uint32_t a0 = nib(perm, sw0);
+        perm = put(put(perm, sw0, nib(perm, 0)), 0, a0);
+        const uint32_t a1 = nib(perm, sw1);
+        perm = put(put(perm, sw1, nib(perm, 1)), 1, a1);
+    }
+    if (KC <= 10 && nlines <= 10) {
+        // the rank of each line among slots 2 .. 9, by all pairs (no branches)
+        constexpr int R = 8;
+        float q[R];
+        int at[R];
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            q[u] = u + 2 < nlines ? pen[(u + 2) * 32] : -CUDART_INF_F;
+            at[u] = 2;
+        }
+#pragma unroll
+        for (int u = 0; u < R; ++u)
+#pragma unroll
+            for (int w = u + 1; w < R; ++w) {
+                if (q[w] > q[u]) ++at[u];
+                else ++at[w];
+            }
+        float4 l[R];
+#pragma unroll
+        for (int u = 0; u < R; ++u) l[u] = L[(u + 2) * 32];
+        const uint64_t was = perm;
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            L[at[u] * 32] = l[u];
+            pen[at[u] * 32] = q[u];
+            if (MODE == MODE_RECORD) perm = put(perm, at[u], nib(was, u + 2));
+        }
+    } else if (nlines <= 16) {   // insertion sort
+        for (int m = 3; m < nlines; ++m) {
+            const float4 e = L[m * 32];
+            const float pe = pen[m * 32];
+            const uint32_t em = MODE == MODE_RECORD ? nib(perm, m) : 0u;
+            int at = m;
+            while (at > 2 && pen[(at - 1) * 32] < pe) {
+                L[at * 32] = L[(at - 1) * 32];
+                pen[at * 32] = pen[(at - 1) * 32];
+                if (MODE == MODE_RECORD) perm = put(perm, at, nib(perm, at - 1));
+                --at;
+            }
+            L[at * 32] = e;
+            pen[at * 32] = pe;
+            if (MODE == MODE_RECORD) perm = put(perm, at, em);
+        }
+    }
+
+    // ---- velocity LP, least-penetration fallback ----
+    float vx, vy, tstar;
+    uint32_t act = 0u;
+    int work = 0;
+    const int infeasible =
+        solve_velocity(L, 32, nlines, vmax, vp.x, vp.y, v.x, v.y,
+                       [&](int i, float4) { return pen[i * 32]; }, vx, vy, tstar, work, act);
+
+    // ---- integrate ----
+    const float2 pn = make_float2(__fadd_rn(p.x, __fmul_rn(sc.dt, vx)),
+                                  __fadd_rn(p.y, __fmul_rn(sc.dt, vy)));
+    const int w = out.caller_order ? o : s;
+    out.vel[w] = make_float2(vx, vy);
+    out.pos[w] = pn;
+    if (out.hint != nullptr) {
+        out.hint[s] = (uint32_t)o;
+        if (s == 0) *out.hint_ok = 1;
+    }
+    if (out.key != nullptr) {
+        // bin the new position for the next step (as the binning kernel's
+        // cell-key phase does on a call's first step)
+        const int ncx = cell_axis(pn.x, sc.origin_x, sc.inv_cell_x, sc.nx);
+        const int ncy = cell_axis(pn.y, sc.origin_y, sc.inv_cell_y, sc.ny);
+        const uint32_t c = (uint32_t)(sc.cell_off + ncy * sc.nx + ncx);
+        out.key[s] = c;
+        out.slot[s] = atomicAdd(out.count + c, 1u);
+    }
+    if (dbg.spos != nullptr) dbg.spos[o] = p;
+    if (dbg.svel != nullptr) dbg.svel[o] = v;
+    if (dbg.vnew != nullptr) dbg.vnew[o] = make_float2(vx, vy);
+    if (MODE == MODE_RECORD && dbg.act != nullptr) {
+        const int nl = act_nlines(act);
+        for (int m = 0; m < nl; ++m) {
+            // the LP's line index in the neighbour order
+            int li = act_line(act, m);
+            if (nlines <= 16) {
+                li = (int)nib(perm, li);
+            } else {   // undo the two swaps
+                li = li == 1 ? sw1 : (li == sw1 ? 1 : li);
+                li = li == 0 ? sw0 : (li == sw0 ? 0 : li);
+            }
+            act = (act & ~(31u << (8 + 8 * m))) | ((uint32_t)li << (8 + 8 * m));
+            act |= ((capbits >> li) & 1u) << (13 + 8 * m);
+            act |= ((ovbits >> li) & 1u) << (14 + 8 * m);
+        }
+        dbg.act[o] = act;
+    }
+    if (dbg.cell != nullptr) dbg.cell[o] = cy * sc.nx + cx;
+    if (dbg.cnt != nullptr) dbg.cnt[o] = cnt;
+    if (dbg.flags != nullptr) dbg.flags[o] = (uint8_t)(infeasible | (any_overlap ? 4 : 0));
+    if (dbg.tstar != nullptr) dbg.tstar[o] = tstar;
+}
+
+}  // namespace orca

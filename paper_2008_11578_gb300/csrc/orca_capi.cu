@@ -24,6 +24,7 @@
 
 #include "orca.h"
 #include "orca_adjoint.cuh"
+#include "orca_agent_solve.cuh"
 #include "orca_cluster_bin.cuh"
 #include "orca_step_kernels.cuh"
 #include "orca_warp_solve.cuh"
@@ -218,34 +219,38 @@ bool kinematic(const orca_params* p) {
     return p->vehicle_turn_rate > 0.0f || p->vehicle_accel > 0.0f;
 }
 
+// Neighbour slots of the per-thread solve kernel: the smallest of its
+// compiled sizes that holds k (10 is the method's usual neighbour count).
+int neighbor_slots(int k) { return k <= 10 ? 10 : (k <= 16 ? 16 : 32); }
+
+size_t agent_smem(int k, bool kin, int block) {
+    const int kl = neighbor_slots(k) + (kin ? kKinLines : 0);
+    return (size_t)agent_units(kl) * block * sizeof(float4);
+}
+
 // More than 48 KB of dynamic shared memory needs an explicit opt-in, set
 // once per scene/batch on its device (outside any stream capture).
+template <class K>
+void allow_smem(cudaError_t& e, K kernel, size_t smem) {
+    if (e == cudaSuccess && smem > 48 * 1024)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 template <class SRC>
-cudaError_t prepare_solve(size_t smem) {
-    if (smem <= 48 * 1024) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(solve_kernel<SRC, MODE_PLAIN>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(solve_kernel<SRC, MODE_COUNT>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(solve_kernel<SRC, MODE_RECORD>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(solve_kernel<SRC, MODE_PLAIN, LP_WORK_UNITS>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(solve_kernel<SRC, MODE_PLAIN, LP_ENUMERATION>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(solve_kernel<SRC, MODE_PLAIN, LP_WARP>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(solve_kernel<SRC, MODE_CHECK>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t prepare_solve(size_t smem, size_t smem_agent) {
+    cudaError_t e = cudaSuccess;
+    allow_smem(e, solve_kernel<SRC, MODE_COUNT, LP_INCREMENTAL>, smem);
+    allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_WORK_UNITS>, smem);
+    allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_ENUMERATION>, smem);
+    allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_WARP>, smem);
+    allow_smem(e, solve_kernel<SRC, MODE_CHECK, LP_INCREMENTAL>, smem);
+    // (10 and 16 neighbour slots stay below 48 KB)
+    allow_smem(e, agent_solve_kernel<SRC, MODE_PLAIN, 32>, smem_agent);
+    allow_smem(e, agent_solve_kernel<SRC, MODE_RECORD, 32>, smem_agent);
     return e;
 }
 
+// The comparison LP schemes, the counting and the checked variant.
 template <class SRC>
 void launch_solve(int mode, int grid, int block, size_t smem, cudaStream_t st, int n, SRC src,
                   const float2* pos, const float2* vel, const uint2* aux, const uint32_t* start,
@@ -255,13 +260,27 @@ void launch_solve(int mode, int grid, int block, size_t smem, cudaStream_t st, i
     solve_kernel<SRC, M, W><<<grid, block, smem, st>>>(n, src, pos, vel, aux, start, ain, vpd, \
                                                         out, dbg, counters, err)
     if (mode == MODE_COUNT) ORCA_SOLVE(MODE_COUNT, LP_INCREMENTAL);
-    else if (mode == MODE_RECORD) ORCA_SOLVE(MODE_RECORD, LP_INCREMENTAL);
     else if (mode == MODE_WORK_UNITS) ORCA_SOLVE(MODE_PLAIN, LP_WORK_UNITS);
     else if (mode == MODE_ENUMERATION) ORCA_SOLVE(MODE_PLAIN, LP_ENUMERATION);
     else if (mode == MODE_WARP_LP) ORCA_SOLVE(MODE_PLAIN, LP_WARP);
-    else if (mode == MODE_CHECK) ORCA_SOLVE(MODE_CHECK, LP_INCREMENTAL);
-    else ORCA_SOLVE(MODE_PLAIN, LP_INCREMENTAL);
+    else ORCA_SOLVE(MODE_CHECK, LP_INCREMENTAL);
 #undef ORCA_SOLVE
+}
+
+template <class SRC, int MODE>
+void launch_agent_solve(int k, bool kin, int grid, int block, cudaStream_t st, int n, SRC src,
+                        const float2* pos, const float2* vel, const uint2* aux,
+                        const uint32_t* start, AgentIn ain, const float2* vpd, StepOut out,
+                        DebugOut dbg, int* err) {
+    const int kc = neighbor_slots(k), kl = kc + (kin ? kKinLines : 0);
+    const size_t smem = agent_smem(k, kin, block);
+#define ORCA_AGENT_SOLVE(KC)                                                              \
+    agent_solve_kernel<SRC, MODE, KC><<<grid, block, smem, st>>>(                         \
+        n, kl, src, pos, vel, aux, start, ain, vpd, out, dbg, err)
+    if (kc == 10) ORCA_AGENT_SOLVE(10);
+    else if (kc == 16) ORCA_AGENT_SOLVE(16);
+    else ORCA_AGENT_SOLVE(32);
+#undef ORCA_AGENT_SOLVE
 }
 
 // The kernel may be set up while the one before it in the stream still runs
@@ -298,7 +317,9 @@ struct Pipeline {
     orca_agents agents;
     int n;
     int ncells;
-    int kcap;
+    int kmax;         // largest k
+    bool kin;         // vehicles have kinematic limits
+    int kcap;         // lines at most
     int block;
     int n_scenes;
     unsigned flags;   // orca_params.debug_flags
@@ -336,16 +357,21 @@ int step_mode(const Pipeline& P) {
 }
 
 // Largest scene solved with one warp per agent.  One thread per agent takes
-// the length of a thread's serial chain however few agents there are (51 us a
-// launch at 1k to 16k agents with k = 10, 217-233 us with k = 32); a warp's
-// chain is 14 us (45 us at 8k agents with k = 32), but the warps of a larger
-// scene queue (2.2 ns an agent with k = 10, 4.2 with k = 32).  The two meet
-// near 22,000 and 55,000 agents (at 24,000: 57 us against 55 us).
-constexpr int kWarpSolveMax = 20480, kWarpSolveMaxWide = 49152;   // up to 16 lines, more
+// the length of a thread's serial chain however few agents there are (44 us a
+// launch at 12,000 agents with k = 10, 75 us with k = 16, 254 us at 32,000
+// with k = 32); a warp's chain is 14 us, but the warps of a larger scene queue
+// (2.4 ns an agent with k = 10, 2.7 with 16, 4.1 with 32).  Per thread / per
+// warp: k = 10 at 16,000 agents 44 / 42 us, at 20,000 47 / 49; k = 16 at 24,000
+// 79 / 67, at 32,000 82 / 85; k = 17 at 64,000 176 / 170, at 250,000 553 / 628;
+// k = 20 at 64,000 227 / 186, at 250,000 656 / 686; from k = 24 the warp is
+// ahead at every size (250,000 agents: 797 / 776 us, with k = 32 1143 / 1030).
+int warp_solve_max(int k) {
+    return k <= 10 ? 18432 : k <= 16 ? 28672 : k < 24 ? 131072 : INT_MAX;
+}
 
 bool solve_by_warp(const Pipeline& P, int mode) {
     return (mode == MODE_PLAIN || mode == MODE_RECORD) && P.kcap <= 32 &&
-           P.n <= (P.kcap <= 16 ? kWarpSolveMax : kWarpSolveMaxWide);
+           P.n <= warp_solve_max(P.kmax);
 }
 
 // Largest scene binned by a cluster.  Against bin_kernel (first step of a call
@@ -460,6 +486,14 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
         if (by_warp)
             launch_warp_solve(mode, wgrid, sb, st, n, src, B.pos1, B.vel1, B.aux[cur], B.start,
                               ain, vpd, out, dbg_for(t), B.err);
+        else if (mode == MODE_RECORD)
+            launch_agent_solve<SRC, MODE_RECORD>(P.kmax, P.kin, sgrid, sb, st, n, src, B.pos1,
+                                                 B.vel1, B.aux[cur], B.start, ain, vpd, out,
+                                                 dbg_for(t), B.err);
+        else if (mode == MODE_PLAIN)
+            launch_agent_solve<SRC, MODE_PLAIN>(P.kmax, P.kin, sgrid, sb, st, n, src, B.pos1,
+                                                B.vel1, B.aux[cur], B.start, ain, vpd, out,
+                                                dbg_for(t), B.err);
         else
             launch_solve(mode, sgrid, sb, smem, st, n, src, B.pos1, B.vel1, B.aux[cur], B.start,
                          ain, vpd, out, dbg_for(t), P.counters, B.err);
@@ -535,8 +569,9 @@ cudaError_t cluster_max(int* out) {
 
 int prepare(Pipeline& P) {
     const size_t smem = solve_smem(P);
-    cudaError_t e = P.n_scenes == 0 ? prepare_solve<OneScene>(smem)
-                                    : prepare_solve<ManyScenes>(smem);
+    const size_t smem_agent = agent_smem(P.kmax, P.kin, P.block);
+    cudaError_t e = P.n_scenes == 0 ? prepare_solve<OneScene>(smem, smem_agent)
+                                    : prepare_solve<ManyScenes>(smem, smem_agent);
     if (e == cudaSuccess)
         e = P.n_scenes == 0 ? bin_grid_max<OneScene>(&P.bin_grid_max)
                             : bin_grid_max<ManyScenes>(&P.bin_grid_max);
@@ -620,14 +655,16 @@ int launch_graph(Pipeline& P, cudaStream_t st) {
     return cuda_status(cudaGraphLaunch(P.graph, st));
 }
 
-void init_pipeline(Pipeline& P, const orca_agents* agents, int ncells, int kcap, int block,
+void init_pipeline(Pipeline& P, const orca_agents* agents, int ncells, int kmax, bool kin, int block,
                    int n_scenes, const Layout& lay, void* workspace, int k_stride,
                    unsigned flags) {
     P.agents = *agents;
     P.flags = flags;
     P.n = agents->n_agents;
     P.ncells = ncells;
-    P.kcap = kcap;
+    P.kmax = kmax;
+    P.kin = kin;
+    P.kcap = kcap_for(kmax, kin);
     P.block = block ? block : 128;
     P.n_scenes = n_scenes;
     P.lay = lay;
@@ -837,7 +874,7 @@ int orca_scene_create(const orca_params* params, const orca_agents* agents, void
     orca_scene* s = new (std::nothrow) orca_scene;
     if (!s) return ORCA_ERR_CAPACITY;
     s->params = *params;
-    init_pipeline(s->p, agents, (int)ncells, kcap_for(params->max_neighbors, kinematic(params)),
+    init_pipeline(s->p, agents, (int)ncells, params->max_neighbors, kinematic(params),
                   params->block_size, 0, lay, workspace, params->max_neighbors,
                   params->debug_flags);
     s->p.one = scene_dev(params, 0, s->p.n, 0);
@@ -1218,7 +1255,7 @@ int orca_batch_create(const orca_params* params, int n_scenes, const int* offset
     if (!b) return ORCA_ERR_CAPACITY;
     b->n_scenes = n_scenes;
     b->kmax = kmax;
-    init_pipeline(b->p, agents, (int)ncells, kcap_for(kmax, kin), params[0].block_size, n_scenes, lay,
+    init_pipeline(b->p, agents, (int)ncells, kmax, kin, params[0].block_size, n_scenes, lay,
                   workspace, kmax, params[0].debug_flags);
     bool ok = cudaMemset(b->p.buf.err, 0, 16) == cudaSuccess &&
               cudaMemset(b->p.buf.count, 0, (size_t)ncells * 4) == cudaSuccess &&
@@ -1342,7 +1379,7 @@ extern "C" int orca_step_noalloc(const orca_params* params, const orca_agents* a
 
     // a pipeline over the scratch area, held on the host stack
     Pipeline P;
-    init_pipeline(P, agents, (int)ncells, kcap_for(params->max_neighbors, kinematic(params)),
+    init_pipeline(P, agents, (int)ncells, params->max_neighbors, kinematic(params),
                   params->block_size,
                   0, L, w, params->max_neighbors, params->debug_flags);
     P.one = scene_dev(params, 0, n, 0);

@@ -433,9 +433,11 @@ __device__ __forceinline__ void pair_bound(const PlanePair& q, const PairLine& b
     num = __fsub_rn(q.beta, mul_add(q.ay, b.bpy, q.ax, b.bpx));
 }
 
+// cof(i, line): det(d, P - s) of line i.
+template <class COF>
 __device__ __forceinline__ float lp3_min_penetration(const float4* __restrict__ L, int stride,
                                                      int n, float vmax, float sx, float sy,
-                                                     float& vx, float& vy, int& work,
+                                                     COF cof, float& vx, float& vy, int& work,
                                                      uint32_t& act, bool* fallback = nullptr) {
     const float tol = lp_tol(vmax);
     float4 l0 = L[0];
@@ -448,12 +450,12 @@ __device__ __forceinline__ float lp3_min_penetration(const float4* __restrict__ 
         if (penetration(li, vx, vy) <= t) continue;
         const float nix = -li.w, niy = li.z;   // objective: maximise n_i . v
         float cx = __fmul_rn(vmax, nix), cy = __fmul_rn(vmax, niy);
-        const float ci = penetration(li, sx, sy);   // det(d, P - s)
+        const float ci = cof(i, li);
         uint32_t ai = act_pack(ACT_VERTEX, true, 1, i, 0, 0);
         for (int j = 0; j < i; ++j) {
             ++work;
             const float4 lj = L[j * stride];
-            const PlanePair q = plane_pair(li, ci, lj, penetration(lj, sx, sy));
+            const PlanePair q = plane_pair(li, ci, lj, cof(j, lj));
             // tested before the bisector is built
             if (!plane_above(q, cx, cy, sx, sy)) continue;
             if (q.a2 <= 1e-12f) continue;   // same direction: one plane dominates
@@ -468,7 +470,7 @@ __device__ __forceinline__ float lp3_min_penetration(const float4* __restrict__ 
             for (int jj = 0; jj < j; ++jj) {
                 work += 2;   // a bisector and a 1D bound
                 const float4 lk = L[jj * stride];
-                const PlanePair k = plane_pair(li, ci, lk, penetration(lk, sx, sy));
+                const PlanePair k = plane_pair(li, ci, lk, cof(jj, lk));
                 if (k.a2 <= 1e-12f) continue;        // same direction
                 float den, num;
                 pair_bound(k, b, den, num);
@@ -606,17 +608,18 @@ __device__ __forceinline__ bool valley_tie_break(const float4* __restrict__ L, i
 // feasible problems such as f = 0 half-planes all through the agent's own
 // velocity on the speed circle.  In dense crowds most agents take the first
 // branch, which saves their 2D LP.
+template <class COF>
 __device__ __forceinline__ int solve_velocity(const float4* __restrict__ L, int stride, int n,
                                               float vmax, float vpx, float vpy, float sx,
-                                              float sy, float& vx, float& vy, float& tstar,
-                                              int& work, uint32_t& act) {
+                                              float sy, COF cof, float& vx, float& vy,
+                                              float& tstar, int& work, uint32_t& act) {
     tstar = 0.0f;
     if (n == 0) return lp2_project(L, stride, n, vmax, vpx, vpy, vx, vy, work, act) == n ? 0 : 1;
     float v3x, v3y;
     uint32_t act3;
     bool fallback = false;
     const float t3 =
-        lp3_min_penetration(L, stride, n, vmax, sx, sy, v3x, v3y, work, act3, &fallback);
+        lp3_min_penetration(L, stride, n, vmax, sx, sy, cof, v3x, v3y, work, act3, &fallback);
     if ((t3 <= 0.1f * lp_tol(vmax) || fallback) &&
         lp2_project(L, stride, n, vmax, vpx, vpy, vx, vy, work, act) == n)
         return 0;
@@ -698,7 +701,9 @@ __device__ __forceinline__ int solve_velocity_work_units(const float4* __restric
     bool live = true;
     if (n > 0) {
         bool fallback = false;
-        t3 = lp3_min_penetration(L, B, n, vmax, sx, sy, v3x, v3y, work, act, &fallback);
+        t3 = lp3_min_penetration(
+            L, B, n, vmax, sx, sy, [&](int, float4 l) { return penetration(l, sx, sy); }, v3x, v3y,
+            work, act, &fallback);
         live = !(t3 > 0.1f * tol && !fallback);
     }
     for (int i = 0; i < kmax; ++i) {

@@ -62,6 +62,8 @@ def test_exact_ties():
     _both(s)
 
 
-@pytest.mark.parametrize("n", [20480, 20481])
-def test_both_sides_of_the_dispatch(n):
-    _both(_moving(scenes.open_square(n, 225.0, seed=73), 6), 1)
+@pytest.mark.parametrize("n,k", [(18432, 10), (18433, 10), (28673, 16), (30000, 30)])
+def test_both_sides_of_the_dispatch(n, k):
+    s = _moving(scenes.open_square(n, (n / 0.4) ** 0.5, seed=73), 6)
+    s.params.max_neighbors = k
+    _both(s, 1)
