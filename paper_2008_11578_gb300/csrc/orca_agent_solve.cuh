@@ -58,6 +58,7 @@ agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
                    const float2* __restrict__ vpd, StepOut out, DebugOut dbg,
                    int* __restrict__ err) {
     extern __shared__ float4 smem_lines[];
+    wait_for_primary();
     // after a binning kernel that gave up or found inconsistent counts the
     // sorted state is not valid: leave everything as it is (the status call
     // reports the error)

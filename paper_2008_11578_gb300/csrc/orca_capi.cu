@@ -267,22 +267,6 @@ void launch_solve(int mode, int grid, int block, size_t smem, cudaStream_t st, i
 #undef ORCA_SOLVE
 }
 
-template <class SRC, int MODE>
-void launch_agent_solve(int k, bool kin, int grid, int block, cudaStream_t st, int n, SRC src,
-                        const float2* pos, const float2* vel, const uint2* aux,
-                        const uint32_t* start, AgentIn ain, const float2* vpd, StepOut out,
-                        DebugOut dbg, int* err) {
-    const int kc = neighbor_slots(k), kl = kc + (kin ? kKinLines : 0);
-    const size_t smem = agent_smem(k, kin, block);
-#define ORCA_AGENT_SOLVE(KC)                                                              \
-    agent_solve_kernel<SRC, MODE, KC><<<grid, block, smem, st>>>(                         \
-        n, kl, src, pos, vel, aux, start, ain, vpd, out, dbg, err)
-    if (kc == 10) ORCA_AGENT_SOLVE(10);
-    else if (kc == 16) ORCA_AGENT_SOLVE(16);
-    else ORCA_AGENT_SOLVE(32);
-#undef ORCA_AGENT_SOLVE
-}
-
 // The kernel may be set up while the one before it in the stream still runs
 // (it waits for that one's end itself, see wait_for_primary).
 cudaLaunchAttribute programmatic_launch() {
@@ -290,6 +274,29 @@ cudaLaunchAttribute programmatic_launch() {
     a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     a.val.programmaticStreamSerializationAllowed = 1;
     return a;
+}
+
+template <class SRC, int MODE>
+void launch_agent_solve(int k, bool kin, bool early, int grid, int block, cudaStream_t st,
+                        int n, SRC src,
+                        const float2* pos, const float2* vel, const uint2* aux,
+                        const uint32_t* start, AgentIn ain, const float2* vpd, StepOut out,
+                        DebugOut dbg, int* err) {
+    const int kc = neighbor_slots(k), kl = kc + (kin ? kKinLines : 0);
+    const size_t smem = agent_smem(k, kin, block);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1] = {programmatic_launch()};
+    cfg.attrs = attr;
+    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg,
+                       kc == 10   ? agent_solve_kernel<SRC, MODE, 10>
+                       : kc == 16 ? agent_solve_kernel<SRC, MODE, 16>
+                                  : agent_solve_kernel<SRC, MODE, 32>,
+                       n, kl, src, pos, vel, aux, start, ain, vpd, out, dbg, err);
 }
 
 template <class SRC>
@@ -462,6 +469,12 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
     const bool by_warp = solve_by_warp(P, mode);
     ClusterShape shape{0, 0};
     const int nb = bin_cluster(P, &shape);
+    // The per-thread solve kernel is set up during the binning only when its
+    // blocks go over more than one wave: placed while the binning blocks still
+    // hold their SMs, the blocks of a smaller grid crowd on the SMs that free
+    // first (65,000 agents: 80 us a step without, 91 with; 250,000: 638 and
+    // 617 us for four steps, the second with the shorter grid barrier).
+    const bool early = sgrid > 2 * P.bin_grid_max;
     const int wgrid = (int)(((long long)n * 32 + sb - 1) / sb);
     // NVTX ranges (host side: the enqueue of each step and its two kernels)
     nvtxRangePushA("orca_step");
@@ -487,11 +500,11 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
             launch_warp_solve(mode, wgrid, sb, st, n, src, B.pos1, B.vel1, B.aux[cur], B.start,
                               ain, vpd, out, dbg_for(t), B.err);
         else if (mode == MODE_RECORD)
-            launch_agent_solve<SRC, MODE_RECORD>(P.kmax, P.kin, sgrid, sb, st, n, src, B.pos1,
+            launch_agent_solve<SRC, MODE_RECORD>(P.kmax, P.kin, early, sgrid, sb, st, n, src, B.pos1,
                                                  B.vel1, B.aux[cur], B.start, ain, vpd, out,
                                                  dbg_for(t), B.err);
         else if (mode == MODE_PLAIN)
-            launch_agent_solve<SRC, MODE_PLAIN>(P.kmax, P.kin, sgrid, sb, st, n, src, B.pos1,
+            launch_agent_solve<SRC, MODE_PLAIN>(P.kmax, P.kin, early, sgrid, sb, st, n, src, B.pos1,
                                                 B.vel1, B.aux[cur], B.start, ain, vpd, out,
                                                 dbg_for(t), B.err);
         else
