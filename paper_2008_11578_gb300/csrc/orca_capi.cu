@@ -838,6 +838,20 @@ struct ReplayDebug {
     }
 };
 
+// The adjoint kernel of one step: four lanes per agent.
+template <class... ARGS>
+void launch_adjoint(cudaStream_t st, int n, ARGS... args) {
+    constexpr int kThreads = 128;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(((long long)n * 4 + kThreads - 1) / kThreads));
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1] = {programmatic_launch()};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, adjoint_kernel, n, args...);
+}
+
 }  // namespace
 
 struct orca_batch {
@@ -1117,7 +1131,6 @@ int orca_adjoint(orca_scene* s, int n_steps, int ckpt_every, const float* vpref_
     const AgentIn ain{(const float2*)A.goal, A.max_speed, A.route, (const float2*)A.waypoints,
                       A.n_waypoints, A.wp_idx};
     int nx = 0, cu = 1, sp = 2;
-    const int ab = 128, ag = (n + ab - 1) / ab;
     for (int seg = L.n_ck - 1; seg >= 0; --seg) {
         const int t0 = seg * ckpt_every;
         const int t1 = std::min(n_steps, t0 + ckpt_every);
@@ -1135,8 +1148,8 @@ int orca_adjoint(orca_scene* s, int n_steps, int ckpt_every, const float* vpref_
             const size_t o = (size_t)(t - t0) * n;
             const size_t tn = (size_t)t * n;
             // the kernel reads the scene's radius/type in caller order
-            adjoint_kernel<<<ag, ab, 0, stm>>>(
-                n, s->p.one, rec.r_pos + o, rec.r_vel + o, A.radius, A.type,
+            launch_adjoint(
+                stm, n, s->p.one, rec.r_pos + o, rec.r_vel + o, A.radius, A.type,
                 rec.r_nbr + o * rec.k, rec.k, rec.r_act + o, rec.r_wp ? rec.r_wp + o : nullptr,
                 rec.r_vnew + o, ain, vpref_delta ? (const float2*)vpref_delta + tn : nullptr,
                 bp[nx], bv[nx], dl_dvel_traj ? (const float2*)dl_dvel_traj + tn : nullptr,
@@ -1208,9 +1221,8 @@ int orca_step_vjp(orca_scene* s, void* adj_ws, size_t adj_bytes, const float* po
     enqueue_steps(R, OneScene{R.one}, 1, vpref_delta, stm, rec, MODE_RECORD);
     const AgentIn ain{(const float2*)A.goal, A.max_speed, A.route, (const float2*)A.waypoints,
                       A.n_waypoints, A.wp_idx};
-    const int ab = 128, ag = (n + ab - 1) / ab;
-    adjoint_kernel<<<ag, ab, 0, stm>>>(
-        n, s->p.one, rec.r_pos, rec.r_vel, A.radius, A.type, rec.r_nbr, rec.k, rec.r_act,
+    launch_adjoint(
+        stm, n, s->p.one, rec.r_pos, rec.r_vel, A.radius, A.type, rec.r_nbr, rec.k, rec.r_act,
         rec.r_wp, rec.r_vnew, ain, (const float2*)vpref_delta, (const float2*)dl_dpos_next,
         (const float2*)dl_dvel_next, nullptr, bp[1], bv[1], bp[2], bv[2],
         (float2*)dl_dvpref_delta, (float2*)dl_dwaypoints, s->p.buf.err);

@@ -74,7 +74,8 @@ __device__ __forceinline__ bool leg_left(float pax, float pay, float pbx, float 
     return d64 > 0.0;
 }
 
-// Squared leg length |q|^2 - rho^2 of the velocity obstacle.  For a pair
+// Squared leg length |q|^2 - rho^2 of the velocity obstacle; l2 is the plain
+// difference qq - rho^2, which stands except near touching.  For a pair
 // close to touching, the FP32 difference of two nearly equal squares keeps
 // only a few correct bits (|q|^2 = 1.000038 against rho^2 = 1 loses three
 // digits), and the leg direction inherits that error.  There it is redone
@@ -87,8 +88,7 @@ __device__ __forceinline__ bool leg_left(float pax, float pay, float pbx, float 
 // result is the exact value up to one final rounding and a few units of
 // 2^-47 rho^2 (as accurate as an FP64 evaluation, without the FP64 pipe).
 __device__ __forceinline__ float leg_l2(float qx, float qy, float ra, float rb, float qq,
-                                        float rho2) {
-    float l2 = __fsub_rn(qq, rho2);
+                                        float l2) {
     if (l2 < 0.015625f * qq) {
         // qx^2 = px + ex, qy^2 = py + ey, s^2 = ps + es exactly
         const float px = __fmul_rn(qx, qx), ex = __fmaf_rn(qx, qx, -px);
@@ -147,7 +147,8 @@ __device__ __forceinline__ float4 orca_line(float pax, float pay, float vax, flo
         } else {
             // legs
             const float qq = mul_add(qx, qx, qy, qy);
-            const float l = sqrtf(fmaxf(leg_l2(qx, qy, ra, rb, qq, rho2), 0.0f));
+            const float l = sqrtf(fmaxf(leg_l2(qx, qy, ra, rb, qq, __fsub_rn(qq, rho2)),
+                                        0.0f));
             const bool left = leg_left(pax, pay, pbx, pby, vax, vay, vbx, vby);
             const float iq = 1.0f / qq;
             if (left) {
