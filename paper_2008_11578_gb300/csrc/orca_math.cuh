@@ -124,52 +124,24 @@ __device__ __forceinline__ float4 orca_line(float pax, float pay, float vax, flo
                                             float ra, float pbx, float pby, float vbx,
                                             float vby, float rb, float f, float inv_tau,
                                             float inv_dt, bool overlap, bool& cap) {
-    cap = false;
     const float qx = __fsub_rn(pbx, pax), qy = __fsub_rn(pby, pay);
     const float wrx = __fsub_rn(vax, vbx), wry = __fsub_rn(vay, vby);
     const float rho = __fadd_rn(ra, rb);
+    const float rho2 = __fmul_rn(rho, rho);
+    // an overlapping pair takes the circle of dt instead of tau
+    const float inv_t = overlap ? inv_dt : inv_tau;
+    const float wx = __fmaf_rn(-qx, inv_t, wrx), wy = __fmaf_rn(-qy, inv_t, wry);
+    const float wq = mul_add(wx, qx, wy, qy);
+    const float ww = mul_add(wx, wx, wy, wy);
+    cap = !overlap && wq < 0.0f && __fmul_rn(wq, wq) > __fmul_rn(rho2, ww);
     float ux, uy, dx, dy;
-    if (!overlap) {
-        const float wx = __fmaf_rn(-qx, inv_tau, wrx), wy = __fmaf_rn(-qy, inv_tau, wry);
-        const float wq = mul_add(wx, qx, wy, qy);
-        const float ww = mul_add(wx, wx, wy, wy);
-        const float rho2 = __fmul_rn(rho, rho);
-        if (wq < 0.0f && __fmul_rn(wq, wq) > __fmul_rn(rho2, ww)) {
-            // cut-off circle
-            cap = true;
-            const float wl = sqrtf(ww);
-            const float hx = wx / wl, hy = wy / wl;
-            dx = hy;
-            dy = -hx;
-            const float s = __fmaf_rn(rho, inv_tau, -wl);
-            ux = __fmul_rn(s, hx);
-            uy = __fmul_rn(s, hy);
-        } else {
-            // legs
-            const float qq = mul_add(qx, qx, qy, qy);
-            const float l = sqrtf(fmaxf(leg_l2(qx, qy, ra, rb, qq, __fsub_rn(qq, rho2)),
-                                        0.0f));
-            const bool left = leg_left(pax, pay, pbx, pby, vax, vay, vbx, vby);
-            const float iq = 1.0f / qq;
-            if (left) {
-                dx = __fmul_rn(mul_sub(qx, l, qy, rho), iq);
-                dy = __fmul_rn(mul_add(qx, rho, qy, l), iq);
-            } else {
-                dx = __fmul_rn(-mul_add(qy, rho, qx, l), iq);
-                dy = __fmul_rn(-mul_sub(qy, l, qx, rho), iq);
-            }
-            const float pr = mul_add(wrx, dx, wry, dy);
-            ux = __fmaf_rn(pr, dx, -wrx);
-            uy = __fmaf_rn(pr, dy, -wry);
-        }
-    } else {
-        const float wx = __fmaf_rn(-qx, inv_dt, wrx), wy = __fmaf_rn(-qy, inv_dt, wry);
-        const float wl = sqrtf(mul_add(wx, wx, wy, wy));
+    if (overlap || cap) {
+        const float wl = sqrtf(ww);
         float hx, hy;
         if (wl > 0.0f) {
             hx = wx / wl;
             hy = wy / wl;
-        } else {
+        } else {   // (overlapping pairs only)
             const float ql = sqrtf(mul_add(qx, qx, qy, qy));
             if (ql > 0.0f) {
                 hx = -qx / ql;
@@ -181,9 +153,26 @@ __device__ __forceinline__ float4 orca_line(float pax, float pay, float vax, flo
         }
         dx = hy;
         dy = -hx;
-        const float s = __fmaf_rn(rho, inv_dt, -wl);
+        const float s = __fmaf_rn(rho, inv_t, -wl);
         ux = __fmul_rn(s, hx);
         uy = __fmul_rn(s, hy);
+    } else {
+        // legs
+        const float qq = mul_add(qx, qx, qy, qy);
+        const float l =
+            sqrtf(fmaxf(leg_l2(qx, qy, ra, rb, qq, __fsub_rn(qq, rho2)), 0.0f));
+        const bool left = leg_left(pax, pay, pbx, pby, vax, vay, vbx, vby);
+        const float iq = 1.0f / qq;
+        if (left) {
+            dx = __fmul_rn(mul_sub(qx, l, qy, rho), iq);
+            dy = __fmul_rn(mul_add(qx, rho, qy, l), iq);
+        } else {
+            dx = __fmul_rn(-mul_add(qy, rho, qx, l), iq);
+            dy = __fmul_rn(-mul_sub(qy, l, qx, rho), iq);
+        }
+        const float pr = mul_add(wrx, dx, wry, dy);
+        ux = __fmaf_rn(pr, dx, -wrx);
+        uy = __fmaf_rn(pr, dy, -wry);
     }
     return make_float4(__fmaf_rn(f, ux, vax), __fmaf_rn(f, uy, vay), dx, dy);
 }
