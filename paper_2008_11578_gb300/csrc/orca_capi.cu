@@ -34,6 +34,7 @@ using namespace orca;
 namespace {
 
 constexpr size_t kAlign = 256;
+static_assert(kRemoveBlocks <= kBinGridMax, "the removal's block sums fit the binning's");
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -48,10 +49,9 @@ struct Layout {
 
 Layout make_layout(size_t n, size_t ncells, size_t n_scenes) {
     Layout L{};
-    // block sums of the binning kernel's scan (one per launch block), and of
-    // the agent scan of orca_scene_remove_arrived
-    size_t nb = std::max((std::max(ncells, n) + kScanChunk - 1) / kScanChunk,
-                         (size_t)kBinGridMax);
+    // block sums of the binning kernel's scan (one per launch block) and of the
+    // removal's, with the total (the size is part of orca_workspace_bytes)
+    size_t nb = std::max((std::max(ncells, n) + 4095) / 4096, (size_t)kBinGridMax);
     size_t o = 0;
     auto take = [&](size_t bytes) {
         size_t at = o;
@@ -63,7 +63,7 @@ Layout make_layout(size_t n, size_t ncells, size_t n_scenes) {
     L.start = take((ncells + 1) * 4);
     L.bsum = take((nb + 1) * 4);
     L.key = take(n * 4);
-    L.slot = take((n + 1) * 4);   // + the total of the agent scan
+    L.slot = take((n + 1) * 4);
     L.hint = take(n * 4);
     L.xrank = take(n * 16);
     L.pos0 = take(n * 8);
@@ -990,39 +990,33 @@ int orca_scene_remove_arrived(orca_scene* s, int* n_kept, int32_t* kept_index, v
     const int n = P.n;
     *n_kept = n;
     if (n == 0) return ORCA_OK;
-    if ((size_t)n > (size_t)kScanChunk * 1024 * 16) return ORCA_ERR_CAPACITY;
+    if (n > (1 << 26)) return ORCA_ERR_CAPACITY;
     cudaStream_t st = (cudaStream_t)stream;
     const Buffers& B = P.buf;
     const orca_agents& A = P.agents;
-    const int tb = 256, gb = (n + tb - 1) / tb;
-    const int nb = (n + kScanChunk - 1) / kScanChunk;
-    // keep flags -> exclusive scan (destinations) -> gather into the step
-    // buffers -> copy back to the front of the caller's arrays
-    arrived_kernel<<<gb, tb, 0, st>>>(n, (const float2*)A.pos, (const float2*)A.goal, A.radius,
-                                      A.route, (const float2*)A.waypoints, A.n_waypoints,
-                                      A.wp_idx, B.key);
-    scan_blocks_kernel<<<nb, kScanThreads, 0, st>>>(B.key, B.slot, B.bsum, n);
-    scan_bsum_kernel<<<1, 1024, 0, st>>>(B.bsum, nb);
-    scan_add_kernel<<<(n / 4 + 256) / 256, 256, 0, st>>>(B.slot, B.bsum, n, nb);
-    compact_gather_kernel<<<gb, tb, 0, st>>>(n, B.slot, (const float2*)A.pos, (const float2*)A.vel,
-                                             (const float2*)A.goal, A.radius, A.max_speed, A.type,
-                                             A.route, A.wp_idx, B.pos0, B.vel0, B.pos1, B.vel1,
-                                             B.aux[0], B.aux[1]);
+    // one tile of agents a block, or as many as keep the blocks few
+    const int tb = kRemoveThreads;
+    const int range = std::max(tb, ((n + kRemoveBlocks - 1) / kRemoveBlocks + tb - 1) / tb * tb);
+    const int gb = (n + range - 1) / range;
+    uint32_t* const total = B.bsum + kRemoveBlocks;
+    // kept agents per block -> destinations and gather into the step buffers
+    // -> copy back to the front of the caller's arrays
+    kept_count_kernel<<<gb, tb, 0, st>>>(n, range, (const float2*)A.pos, (const float2*)A.goal,
+                                         A.radius, A.route, (const float2*)A.waypoints,
+                                         A.n_waypoints, A.wp_idx, B.bsum);
+    compact_gather_kernel<<<gb, tb, 0, st>>>(
+        n, range, B.bsum, (const float2*)A.pos, (const float2*)A.vel, (const float2*)A.goal,
+        A.radius, A.max_speed, A.type, A.route, (const float2*)A.waypoints, A.n_waypoints,
+        A.wp_idx, B.pos0, B.vel0, B.pos1, B.vel1, B.aux[0], B.aux[1], total);
     uint32_t kept = 0;
-    if (cudaMemcpyAsync(&kept, B.slot + n, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    if (cudaMemcpyAsync(&kept, total, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return ORCA_ERR_CUDA;
-    if (kept > 0)
-        compact_scatter_kernel<<<((int)kept + tb - 1) / tb, tb, 0, st>>>(
-            (int)kept, B.pos0, B.vel0, B.pos1, B.vel1, B.aux[0], B.aux[1], (float2*)A.pos,
-            (float2*)A.vel, (float2*)A.goal, (float*)A.radius, (float*)A.max_speed,
-            (uint8_t*)A.type, (int32_t*)A.route, A.wp_idx, kept_index);
+    compact_scatter_kernel<<<std::max(1, ((int)kept + tb - 1) / tb), tb, 0, st>>>(
+        (int)kept, B.pos0, B.vel0, B.pos1, B.vel1, B.aux[0], B.aux[1], (float2*)A.pos,
+        (float2*)A.vel, (float2*)A.goal, (float*)A.radius, (float*)A.max_speed, (uint8_t*)A.type,
+        (int32_t*)A.route, A.wp_idx, kept_index, B.err + 1);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
-        return ORCA_ERR_CUDA;
-    // the recorded sorted order names the old indices: bin the next call in
-    // the caller's order
-    if (cudaMemsetAsync(B.err + 1, 0, 4, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
         return ORCA_ERR_CUDA;
     P.n = (int)kept;
     drop_graph(P);   // a graph recorded for the old count is stale

@@ -146,8 +146,4 @@ constexpr int kNumCounters = 13;
 // ERR_BIT_CHECK: a checked step (MODE_CHECK) found a broken invariant.
 enum : int { ERR_BIT_NONFINITE = 1, ERR_BIT_TIMEOUT = 2, ERR_BIT_STATE = 4, ERR_BIT_CHECK = 8 };
 
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 16;
-constexpr int kScanChunk = kScanThreads * kScanItems;   // cells per scan block
-
 }  // namespace orca
