@@ -182,4 +182,56 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     cl.sync();   // no block leaves while another reads its records
 }
 
+// ------------------------------------------------------- no cells at all ----
+// The smallest scenes: the agents sorted by one coordinate (y if by_y), by
+// counting for each agent the keys below its own (equal ones by index).  Every
+// block reads all coordinates, so no block waits for another: one round trip to
+// memory and n / 8 comparisons per lane (eight lanes an agent) in place of the
+// cluster's count, scan, scatter and rank.
+constexpr int kFlatMax = 1024;
+constexpr int kFlatThreads = 256;
+constexpr int kFlatLanes = 8;
+constexpr int kFlatAgents = kFlatThreads / kFlatLanes;   // per block
+
+template <bool FIRST>
+__global__ void __launch_bounds__(kFlatThreads) flat_bin_kernel(BinArgs a, bool by_y) {
+    __shared__ uint32_t keys[kFlatMax];
+    launch_dependents();
+    wait_for_primary();
+    const float2* __restrict__ pos = FIRST ? a.upos : a.pos0;
+    const int tid = (int)threadIdx.x, q = tid % kFlatLanes;
+    const int i = (int)blockIdx.x * kFlatAgents + tid / kFlatLanes;
+    float2 p = make_float2(0.0f, 0.0f), v = p;
+    uint2 ax = make_uint2(0u, 0u);
+    if (i < a.n) {   // (its loads overlap the staging)
+        p = pos[i];
+        if (q == 0) {
+            v = FIRST ? a.uvel[i] : a.vel0[i];
+            ax = FIRST ? aux_pack(a.urad[i], a.utype[i], i) : a.aux0[i];
+        }
+    }
+    for (int j = tid; j < a.n; j += kFlatThreads) {
+        const float2 c = pos[j];
+        keys[j] = x_order_key(by_y ? c.y : c.x);
+    }
+    if (FIRST && q == 0 && i < a.n &&
+        !(isfinite(p.x) && isfinite(p.y) && isfinite(v.x) && isfinite(v.y)))
+        atomicOr(a.err, ERR_BIT_NONFINITE);
+    __syncthreads();
+    const uint32_t own = x_order_key(by_y ? p.y : p.x);
+    uint32_t rank = 0u;
+#pragma unroll 4
+    for (int j = q; j < a.n; j += kFlatLanes) {
+        const uint32_t k = keys[j];
+        rank += (k < own || (k == own && j < i)) ? 1u : 0u;
+    }
+#pragma unroll
+    for (int d = 1; d < kFlatLanes; d <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, d);
+    if (q == 0 && i < a.n) {
+        a.pos1[rank] = p;
+        a.vel1[rank] = v;
+        a.aux1[rank] = ax;
+    }
+}
+
 }  // namespace orca

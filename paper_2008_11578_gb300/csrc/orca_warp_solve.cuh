@@ -12,7 +12,8 @@
 // Bound by the latency of one agent's chain while the scene is small (1,000
 // agents: 51 -> 14 us a launch, about 12,500 cycles an agent: loads 1,600,
 // seed 2,100, scan 1,900, half-planes 1,400, order 900, LP 3,600), then by
-// issue slots (16,000 agents: 51 -> 41 us, 73 % of issue slots busy).
+// issue slots (16,000 agents: 51 -> 40 us, 73 % of issue slots busy; eight
+// blocks an SM 39.7 us, seven 40.9, six 41.0, five 43.0).
 #pragma once
 
 #include "orca_step_kernels.cuh"
@@ -227,9 +228,15 @@ __device__ __forceinline__ int warp_solve_velocity(const float4* L, float4 lj, i
 // one shift of the lanes behind it.  The list is the set of the k smallest
 // keys whatever the order of the candidates, so it equals the per-thread
 // kernel's.
-template <class SRC, int MODE>
-__global__ void __launch_bounds__(128)
-warp_solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* __restrict__ vel,
+//
+// FLAT: the smallest scenes, not binned into cells but sorted by one coordinate
+// (y if by_y, else x): one row of all slots, 16 on either side of the agent
+// seed the list, and both sides go on until the coordinate alone is beyond the
+// bound; the first 32 slots after the seed's are loaded with it, each later 32
+// while the ones before are tested.
+template <class SRC, int MODE, bool FLAT>
+__global__ void __launch_bounds__(128, 8)
+warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos, const float2* __restrict__ vel,
                   const uint2* __restrict__ aux, const uint32_t* __restrict__ cstart, AgentIn ain,
                   const float2* __restrict__ vpd, StepOut out, DebugOut dbg,
                   int* __restrict__ err) {
@@ -278,11 +285,11 @@ warp_solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* 
     unsigned long long key = ~0ull;
     int slot = -1, cnt = 0;
     if (k > 0 && isfinite(p.x) && isfinite(p.y)) {
-        const uint32_t* __restrict__ cs = cstart + sc.cell_off;
         const uint32_t* __restrict__ aux_idx = reinterpret_cast<const uint32_t*>(aux) + 1;
-        const int nx = sc.nx, ny = sc.ny;
         const float R2 = sc.R2;
         const float thr0 = R2 > 0.0f ? __int_as_float(__float_as_int(R2) - 1) : -1.0f;
+        const uint32_t* __restrict__ cs = cstart + sc.cell_off;
+        const int nx = sc.nx, ny = sc.ny;
         const float ch = sc.cell_h, mg = sc.ring_delta * ch;
         const float pry = __fsub_rn(p.y, sc.origin_y);
         auto row_gap2 = [&](int ry) {
@@ -304,51 +311,74 @@ warp_solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* 
             if (ry >= 0 && ry < ny)
                 range = (int)__ldg(cs + (size_t)ry * nx + (q == 0 ? 0 : q == 1 ? nx : cx + q - 2));
         };
-        load_rows();
+        if (!FLAT) load_rows();
         // ---- seed ----
-        // Lanes 0-7 take the own row; the others the rows around it, nearest
-        // slots first, half of them each way.  Dense: 8 each way in the own
-        // row and 4 in the rows next to it.  Sparse (the k-th neighbour is
-        // probably beyond the next row, judged by the agents in the own
-        // column's three cells): 4 in the own row, 3 in two rows on each side.
-        const int i0 = (cy - row0) << 2;
-        int column = __shfl_sync(kFull, range, i0 + 3) - __shfl_sync(kFull, range, i0 + 2);
-        column += __shfl_sync(kFull, range, i0 - 1) - __shfl_sync(kFull, range, i0 - 2);
-        column += __shfl_sync(kFull, range, i0 + 7) - __shfl_sync(kFull, range, i0 + 6);
-        const bool sparse = 3.0f * (float)k * sc.cell_w > 4.5f * (float)column * ch;
-        int off = 0, step = lane & 7, half = 4;   // row offset, place in the row's lanes
-        if (sparse) {
-            if (lane >= 8) {
-                const int u = lane - 8;   // 6 lanes for each of rows -1, +1, -2, +2
-                const int w = u / 6;
-                off = (w & 1 ? 1 : -1) * (1 + (w >> 1));
-                step = u - 6 * w;
-                half = 3;
+        bool sparse = false, left = lane >= 16;
+        int off = 0, step = lane & 15, half = 16;   // row offset, place in the row's lanes
+        int rb = 0, re = n, start = s;
+        float g2s = 0.0f;
+        float2 ahead[2];          // FLAT: the slots after the seed's, rightward and leftward
+        uint32_t ahead_idx[2];
+        auto load = [&](int j, float2& c, uint32_t& oc) {
+            if (j >= 0 && j < n) {
+                c = pos[j];
+                oc = __ldg(aux_idx + 2 * j);
             }
-        } else if (lane < 16) {
-            step = lane;
-            half = 8;
+        };
+        if (FLAT) {
+            load(s + 17 + lane, ahead[0], ahead_idx[0]);
+            load(s - 17 - lane, ahead[1], ahead_idx[1]);
         } else {
-            off = lane < 24 ? -1 : 1;
+            step = lane & 7;
+            half = 4;
+            // Lanes 0-7 take the own row; the others the rows around it, nearest
+            // slots first, half of them each way.  Dense: 8 each way in the own
+            // row and 4 in the rows next to it.  Sparse (the k-th neighbour is
+            // probably beyond the next row, judged by the agents in the own
+            // column's three cells): 4 in the own row, 3 in two rows on each side.
+            const int i0 = (cy - row0) << 2;
+            int column = __shfl_sync(kFull, range, i0 + 3) - __shfl_sync(kFull, range, i0 + 2);
+            column += __shfl_sync(kFull, range, i0 - 1) - __shfl_sync(kFull, range, i0 - 2);
+            column += __shfl_sync(kFull, range, i0 + 7) - __shfl_sync(kFull, range, i0 + 6);
+            sparse = 3.0f * (float)k * sc.cell_w > 4.5f * (float)column * ch;
+            if (sparse) {
+                if (lane >= 8) {
+                    const int u = lane - 8;   // 6 lanes for each of rows -1, +1, -2, +2
+                    const int w = u / 6;
+                    off = (w & 1 ? 1 : -1) * (1 + (w >> 1));
+                    step = u - 6 * w;
+                    half = 3;
+                }
+            } else if (lane < 16) {
+                step = lane;
+                half = 8;
+            } else {
+                off = lane < 24 ? -1 : 1;
+            }
+            left = step >= half;
+            if (left) step -= half;
+            const int ib = i0 + 4 * off;
+            rb = __shfl_sync(kFull, range, ib);
+            re = __shfl_sync(kFull, range, ib + 1);
+            const int bc = __shfl_sync(kFull, range, ib + 2), ec = __shfl_sync(kFull, range, ib + 3);
+            start = off == 0 ? s : min(bc + (int)(fx * (float)(ec - bc)), ec);
+            g2s = off == 0 ? 0.0f : row_gap2(cy + off);
         }
-        const bool left = step >= half;
-        if (left) step -= half;
-        const int ib = i0 + 4 * off;
-        const int rb = __shfl_sync(kFull, range, ib), re = __shfl_sync(kFull, range, ib + 1);
-        const int bc = __shfl_sync(kFull, range, ib + 2), ec = __shfl_sync(kFull, range, ib + 3);
-        const int start = off == 0 ? s : min(bc + (int)(fx * (float)(ec - bc)), ec);
-        const float g2s = off == 0 ? 0.0f : row_gap2(cy + off);
         const int js = left ? start - 1 - step : start + (off == 0 ? 1 : 0) + step;
         const bool in = js >= rb && js < re;
+        // distance along the rows (dx, or dy when sorted by y), its square, d^2
+        auto measure = [&](float2 c, float& along, float& along2) {
+            const float dx = __fsub_rn(c.x, p.x), dy = __fsub_rn(c.y, p.y);
+            const float xx = __fmul_rn(dx, dx), yy = __fmul_rn(dy, dy);
+            along = FLAT && by_y ? dy : dx;
+            along2 = FLAT && by_y ? yy : xx;
+            return __fadd_rn(xx, yy);
+        };
         float ds = CUDART_INF_F, dxs = 0.0f, dxxs = 0.0f;
         uint32_t os = 0u;
         if (in) {
-            const float2 c = pos[js];
             os = __ldg(aux_idx + 2 * js);
-            dxs = __fsub_rn(c.x, p.x);
-            dxxs = __fmul_rn(dxs, dxs);
-            const float dy = __fsub_rn(c.y, p.y);
-            const float d2 = __fadd_rn(dxxs, __fmul_rn(dy, dy));
+            const float d2 = measure(pos[js], dxs, dxxs);
             if (d2 <= thr0) ds = d2;
         }
         const int oj = aux_orig(make_uint2(0u, os));
@@ -438,25 +468,23 @@ warp_solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* 
             if (lane >= k) key = ~0ull;   // pushed out of the list
             update();
         };
-        // candidate at slot j of a row whose y gap^2 is g2: enters the list when
-        // below the bound; returns whether it and all farther ones on its side
-        // are beyond it
-        auto test = [&](bool on, int j, bool lf, float g2) {
+        // candidate c (index word oc) at slot j of a row whose y gap^2 is g2:
+        // enters the list when below the bound; returns whether it and all
+        // farther ones on its side are beyond it
+        auto test_loaded = [&](bool on, int j, bool lf, float g2, float2 c, uint32_t oc) {
             float d2 = CUDART_INF_F, dx = 0.0f, dxx = 0.0f;
-            uint32_t oc = 0u;
-            if (on) {
-                const float2 c = pos[j];
-                oc = __ldg(aux_idx + 2 * j);
-                dx = __fsub_rn(c.x, p.x);
-                dxx = __fmul_rn(dx, dx);
-                const float dy = __fsub_rn(c.y, p.y);
-                d2 = __fadd_rn(dxx, __fmul_rn(dy, dy));
-            }
+            if (on) d2 = measure(c, dx, dxx);
             const unsigned am = __ballot_sync(kFull, on && d2 <= thr_d);
             if (am != 0u)
                 admit(am, ((unsigned long long)__float_as_uint(d2) << 32) |
                               (unsigned)aux_orig(make_uint2(0u, oc)), j);
             return !on || ((lf ? dx < 0.0f : dx > 0.0f) && __fadd_rn(dxx, g2) > thr_d);
+        };
+        auto test = [&](bool on, int j, bool lf, float g2) {
+            float2 c = make_float2(0.0f, 0.0f);
+            uint32_t oc = 0u;
+            if (on) load(j, c, oc);
+            return test_loaded(on, j, lf, g2, c, oc);
         };
         // The seeded rows go on from where their seed ended, 32 slots at a time,
         // on the sides that it left open: a side is finished when a candidate on
@@ -466,6 +494,25 @@ warp_solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* 
         const unsigned my_side = ((1u << half) - 1u) << (lane - step);
         unsigned open = __ballot_sync(kFull,
                                       step == 0 && (fin & my_side) == 0u && g2s <= thr_d);
+        if (FLAT) {
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                const bool lf = side == 1;
+                if ((open & (lf ? 0xffff0000u : 0xffffu)) == 0u) continue;
+                int j = lf ? s - 17 - lane : s + 17 + lane;
+                for (;;) {
+                    const float2 c = ahead[side];
+                    const uint32_t oc = ahead_idx[side];
+                    const int next = lf ? j - 32 : j + 32;
+                    load(next, ahead[side], ahead_idx[side]);
+                    if (__ballot_sync(kFull, test_loaded(j >= 0 && j < n, j, lf, 0.0f, c, oc)) !=
+                        0u)
+                        break;
+                    j = next;
+                }
+            }
+            open = 0u;
+        }
         for (; open != 0u; open &= open - 1u) {
             const int u = __ffs(open) - 1;   // the side's first lane
             const bool lf = __shfl_sync(kFull, left ? 1 : 0, u) != 0;
@@ -479,7 +526,7 @@ warp_solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* 
         }
         // The rows farther out, 16 slots each way at a time; a side ends at the
         // grid edge or at the first row whose y gap is beyond the bound.
-        bool up = true, down = true;
+        bool up = !FLAT, down = !FLAT;
         for (int m = sparse ? 3 : 2; up || down; ++m) {
             const float gd = row_gap2(cy - m), gu = row_gap2(cy + m);
             const int first = gu < gd ? 1 : 0;

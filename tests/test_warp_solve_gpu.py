@@ -54,12 +54,29 @@ def test_vehicle_limits(k):
     _both(s)
 
 
+@pytest.mark.parametrize("tall", [False, True])
+@pytest.mark.parametrize("n,k", [(2, 10), (17, 10), (40, 10), (1023, 32), (1024, 10), (1025, 10)])
+def test_scenes_without_cells(n, k, tall):
+    """The smallest scenes are sorted along the longer side of their box and
+    searched without cells, here also with agents outside the box, some at the
+    same coordinate, and most beyond the neighbour distance."""
+    s = _moving(scenes.open_square(n, 60.0, seed=74 + k), 8)
+    s.params.max_neighbors = k
+    a, b = (0, 1) if tall else (1, 0)
+    s.pos[:, a] *= np.float32(0.2)
+    s.pos[: n // 3, b] = s.pos[0, b]
+    s.pos[n // 2:, b] *= np.float32(9.0)
+    s.params.extent = (12.0, 60.0) if tall else (60.0, 12.0)
+    _both(s, 3)
+
+
 def test_exact_ties():
     """A lattice at rest: equal distances everywhere, equal penetrations."""
     s = scenes.open_square(2500, 40.0, seed=72)
     g = np.stack(np.meshgrid(np.arange(50), np.arange(50)), -1).reshape(-1, 2)
     s.pos = np.ascontiguousarray(0.75 * g, dtype=np.float32)
     _both(s)
+    _both(s.subset(np.arange(900)))
 
 
 @pytest.mark.parametrize("n,k", [(18432, 10), (18433, 10), (28673, 16), (30000, 30)])
