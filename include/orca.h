@@ -111,7 +111,8 @@ extern "C" {
  *                   agent's x, so the row height sets how far beyond the
  *                   k-th nearest neighbour it looks
  *   origin_x/y, grid_nx/ny   grid box; agents outside clamp to edge cells
- *   block_size      threads per block of the solve kernel (0 = 128)
+ *   block_size      threads per block of the solve kernel (0: 128, or 64
+ *                   where its per-thread variant runs in several waves)
  *   debug_flags     ORCA_DEBUG_NONE, or one of ORCA_FLAG_LP_WORK_UNITS,
  *                   ORCA_FLAG_LP_ENUMERATION, ORCA_FLAG_LP_WARP and
  *                   ORCA_DEBUG_CHECKED, and/or ORCA_DEBUG_BARRIER_TIMEOUT
