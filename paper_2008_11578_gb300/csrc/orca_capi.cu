@@ -1096,7 +1096,7 @@ int orca_scene_remove_arrived(orca_scene* s, int* n_kept, int32_t* kept_index, v
     compact_scatter_kernel<<<std::max(1, ((int)kept + tb - 1) / tb), tb, 0, st>>>(
         (int)kept, B.pos0, B.vel0, B.pos1, B.vel1, B.aux[0], B.aux[1], (float2*)A.pos,
         (float2*)A.vel, (float2*)A.goal, (float*)A.radius, (float*)A.max_speed, (uint8_t*)A.type,
-        (int32_t*)A.route, A.wp_idx, kept_index, B.err + 1);
+        (int32_t*)A.route, A.wp_idx, kept_index, (int)kept < n ? B.err + 1 : nullptr);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
         return ORCA_ERR_CUDA;
     P.n = (int)kept;

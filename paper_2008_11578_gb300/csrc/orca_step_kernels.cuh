@@ -522,9 +522,9 @@ __global__ void compact_scatter_kernel(int kept, const float2* __restrict__ t_po
                                        int32_t* __restrict__ kept_index,
                                        int* __restrict__ hint_ok) {
     const int d = blockIdx.x * blockDim.x + threadIdx.x;
-    // the recorded sorted order names the old indices: the next call bins in
-    // the caller's order
-    if (d == 0) *hint_ok = 0;
+    // once an agent has left, the recorded sorted order names old indices: the
+    // next call bins in the caller's order
+    if (d == 0 && hint_ok != nullptr) *hint_ok = 0;
     if (d >= kept) return;
     pos[d] = t_pos[d];
     vel[d] = t_vel[d];
