@@ -619,7 +619,7 @@ def measure_removal(dev, arrive_every=10, reps=3):
     return {"workload": "clusters_1m", "agents": n, "kept": nk, "ms": ms,
             "bytes": alg, "achieved_gbs": alg / (ms / 1e3) / 1e9,
             "frac": alg / (ms / 1e3) / 1e9 / hbm,
-            "kernels": "arrived_kernel, scan kernels, compact_gather_kernel, "
+            "kernels": "kept_count_kernel, compact_gather_kernel, "
                        "compact_scatter_kernel",
             "note": "one call with its host synchronisation (the new count)"}
 

@@ -58,21 +58,26 @@ __device__ __forceinline__ int count_below(const float* v, float x) {
 }
 
 // Interval of a 1D sub-problem after the bounds of the lanes that have one
-// (upper: t <= tt, lower: t >= tt) are merged into [tl, tr]; kl and kr name
-// the first lane that set each end (-1: none did).
-__device__ __forceinline__ void merge_bounds(bool upper, bool lower, float tt, float& tl,
-                                             float& tr, int& kl, int& kr) {
+// (upper: t <= tt, lower: t >= tt) are merged into [tl, tr]; with ACT, kl and kr
+// name the first lane that set each end (-1: none did).  A lane that finds the
+// sub-problem empty (empty) puts the lower end at infinity.
+template <bool ACT>
+__device__ __forceinline__ void merge_bounds(bool upper, bool lower, bool empty, float tt,
+                                             float& tl, float& tr, int& kl, int& kr) {
     const float hi = redux_min(upper ? tt : CUDART_INF_F);
-    const float lo = redux_max(lower ? tt : -CUDART_INF_F);
-    const unsigned mr = __ballot_sync(kFull, upper && tt == hi);
-    const unsigned ml = __ballot_sync(kFull, lower && tt == lo);
-    kr = hi < tr ? __ffs(mr) - 1 : -1;
-    kl = lo > tl ? __ffs(ml) - 1 : -1;
+    const float lo = redux_max(empty ? CUDART_INF_F : (lower ? tt : -CUDART_INF_F));
+    if (ACT) {
+        const unsigned mr = __ballot_sync(kFull, upper && tt == hi);
+        const unsigned ml = __ballot_sync(kFull, lower && tt == lo);
+        kr = hi < tr ? __ffs(mr) - 1 : -1;
+        kl = lo > tl ? __ffs(ml) - 1 : -1;
+    }
     tr = fminf(tr, hi);
     tl = fmaxf(tl, lo);
 }
 
 // lp2_project over the warp: lane j holds line lj (j < n), L the same lines.
+template <bool ACT>
 __device__ __forceinline__ int warp_lp2(const float4* L, float4 lj, int lane, int n, float vmax,
                                         float vpx, float vpy, float& vx, float& vy,
                                         uint32_t& act) {
@@ -93,9 +98,9 @@ __device__ __forceinline__ int warp_lp2(const float4* L, float4 lj, int lane, in
         line_bound(li, lj, den, num);
         const bool on = lane < i;
         const float tt = __fdividef(num, den);
-        if (__any_sync(kFull, on && den == 0.0f && num < -tol)) return i;
-        int kl, kr;
-        merge_bounds(on && den > 0.0f, on && den < 0.0f, tt, tl, tr, kl, kr);
+        int kl = -1, kr = -1;
+        merge_bounds<ACT>(on && den > 0.0f, on && den < 0.0f, on && den == 0.0f && num < -tol, tt,
+                          tl, tr, kl, kr);
         if (tl > tr + tol) return i;
         const float t0 = line_project(li, vpx, vpy, tl, tr, vx, vy);
         const int bound = (t0 > tr) ? kr : ((t0 < tl) ? kl : -2);
@@ -105,6 +110,7 @@ __device__ __forceinline__ int warp_lp2(const float4* L, float4 lj, int lane, in
 }
 
 // lp3_min_penetration over the warp.
+template <bool ACT>
 __device__ __forceinline__ float warp_lp3(const float4* L, float4 lj, int lane, int n, float vmax,
                                           float sx, float sy, float& vx, float& vy, uint32_t& act,
                                           bool& fallback) {
@@ -151,10 +157,10 @@ __device__ __forceinline__ float warp_lp3(const float4* L, float4 lj, int lane, 
             pair_bound(q, b, den, num);
             const bool on = lane < j && !(q.a2 <= 1e-12f);
             const float tt = __fdividef(num, den);
-            const bool bad = __any_sync(kFull, on && den == 0.0f && num > tol);
-            int kl, kr;
-            merge_bounds(on && den < 0.0f, on && den > 0.0f, tt, tl, tr, kl, kr);
-            if (bad || tl > tr + tol) {   // empty only through rounding: keep the point
+            int kl = -1, kr = -1;
+            merge_bounds<ACT>(on && den < 0.0f, on && den > 0.0f, on && den == 0.0f && num > tol,
+                              tt, tl, tr, kl, kr);
+            if (tl > tr + tol) {   // empty only through rounding: keep the point
                 fallback = true;
                 continue;
             }
@@ -175,6 +181,7 @@ __device__ __forceinline__ float warp_lp3(const float4* L, float4 lj, int lane, 
 }
 
 // solve_velocity over the warp.
+template <bool ACT>
 __device__ __forceinline__ int warp_solve_velocity(const float4* L, float4 lj, int lane, int n,
                                                    float vmax, float vpx, float vpy, float sx,
                                                    float sy, float& vx, float& vy, float& tstar,
@@ -183,9 +190,9 @@ __device__ __forceinline__ int warp_solve_velocity(const float4* L, float4 lj, i
     float v3x = 0.0f, v3y = 0.0f, t3 = -CUDART_INF_F;
     uint32_t act3 = 0u;
     bool fallback = false;
-    if (n > 0) t3 = warp_lp3(L, lj, lane, n, vmax, sx, sy, v3x, v3y, act3, fallback);
+    if (n > 0) t3 = warp_lp3<ACT>(L, lj, lane, n, vmax, sx, sy, v3x, v3y, act3, fallback);
     if ((t3 <= 0.1f * lp_tol(vmax) || fallback || n == 0) &&
-        warp_lp2(L, lj, lane, n, vmax, vpx, vpy, vx, vy, act) == n)
+        warp_lp2<ACT>(L, lj, lane, n, vmax, vpx, vpy, vx, vy, act) == n)
         return 0;
     act = act3;
     tstar = t3;
@@ -637,8 +644,8 @@ warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos, con
     // ---- velocity LP, least-penetration fallback ----
     float vx, vy, tstar;
     uint32_t act = 0u;
-    const int infeasible = warp_solve_velocity(W.line, lj, lane, nlines, vmax, vp.x, vp.y, v.x,
-                                               v.y, vx, vy, tstar, act);
+    const int infeasible = warp_solve_velocity<MODE == MODE_RECORD>(
+        W.line, lj, lane, nlines, vmax, vp.x, vp.y, v.x, v.y, vx, vy, tstar, act);
     if (MODE == MODE_RECORD && dbg.act != nullptr) {
         // line indices back in neighbour order, with each line's construction
         const unsigned capbits = __ballot_sync(kFull, cap), ovbits = __ballot_sync(kFull, ov);
