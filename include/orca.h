@@ -237,7 +237,7 @@ int orca_scene_set_solve_events(orca_scene *scene, void *begin, void *end);
 
 /*
  * The same for the binning phase (cell keys, the scan of the cell counts and
- * the scatter into cell order, one cooperative kernel per step): begin and
+ * the scatter into cell order, one kernel per step): begin and
  * end bracket that kernel.  On the first step of a call it also reads the
  * caller's arrays (later steps read the state the solve kernel wrote).
  */

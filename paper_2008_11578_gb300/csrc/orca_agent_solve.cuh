@@ -8,17 +8,19 @@
 // distances differ only in the replaced bits (some 5e-4 of the agents, or
 // lattices) the list is put in order exactly.
 //
-// Bound by issue slots (0.71 of one instruction a cycle per scheduler, 44 % of
-// an instruction's lanes active: the LP's re-solves and the half-planes'
-// constructions differ between the lanes) in large scenes, by one thread's chain
-// in smaller ones.  1M clusters, first step of a call: 454 us with the sorted
-// list in shared memory, 420 with the network and a pass that ranks the admitted
-// slots, 394 with the places carried in the entries, 377-380 with the LP's order
-// by all pairs and the penetrations kept for the LP (65,000-agent shared space:
-// 67, 55, 58, 52).  Of it the row scan takes about 90 us, the network 60, the
-// half-planes 58, the LP 130.  Seven blocks an SM (72 registers) measured 380 us
-// there and 73 us at 130,000 agents, six 403 and 88, eight 377 and 76, nine 396
-// and 79.
+// Bound by issue slots in large scenes (0.74 of one instruction a cycle per
+// scheduler, 57 % of an instruction's lanes active: the LP's re-solves and the
+// half-planes' constructions differ between the lanes; 4 % of the memory's
+// rate), by one thread's chain in smaller ones.  1M clusters, one step: 454 us
+// with the sorted list in shared memory, 420 with the network and a pass that
+// ranks the admitted slots, 394 with the places carried in the entries, 378 with
+// the LP's order by all pairs and the penetrations kept for the LP (the
+// 65,000-agent shared space: 67, 55, 58, 52), 375 with one construction of the
+// cut-off and overlap half-planes, 367 in blocks of two warps.  (The benchmark's
+// 1M crowd after its warm-up steps: 381 -> 304 us.)  Of the 378 the row scan took
+// about 90 us, the network 60, the half-planes 58, the LP 130.  Registers, in the
+// same form: seven blocks of four warps an SM (72) 380 us and 73 us at 130,000
+// agents, six 403 and 88, eight 377 and 76, nine 396 and 79.
 #pragma once
 
 #include "orca_step_kernels.cuh"

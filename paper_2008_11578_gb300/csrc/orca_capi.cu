@@ -1,10 +1,12 @@
 // orca_capi.cu -- the C ABI of liborca (declared in include/orca.h).
 //
 // Host side of the ORCA step: argument validation, workspace layout, and
-// the launch sequence: per step one cooperative binning kernel (on a call's
-// first step it reads the caller's arrays) and the solve kernel (which bins
-// the new positions for the next step, and writes the last step's results
-// straight into the caller's arrays).
+// the launch sequence: per step one binning kernel (on a call's first step it
+// reads the caller's arrays) and one solve kernel (which bins the new positions
+// for the next step where the binning wants it, and writes the last step's
+// results straight into the caller's arrays).  Which of the variants runs depends
+// on the number of agents and on k (solve_by_warp, solve_flat, bin_cluster);
+// their results are the same.
 //
 // A single scene and a batch of independent scenes run the same kernels.  A
 // batch concatenates its scenes' agents (scene 0 first) and their grid cells
@@ -430,8 +432,9 @@ int bin_cluster(const Pipeline& P, ClusterShape* sh) {
     return 0;
 }
 
-// The binning kernel of one step (cooperative launch, grid sized to what is
-// resident at once on this device).  first: from the caller's arrays.
+// The binning kernel of one step: without cells, by one cluster, or the
+// cooperative launch, its grid sized to what is resident at once on this device.
+// first: from the caller's arrays.
 template <class SRC>
 void launch_bin(const Pipeline& P, SRC src, bool first, int cur, bool flat, bool by_y, int nb,
                 ClusterShape sh, cudaStream_t st) {
@@ -488,9 +491,8 @@ void launch_bin(const Pipeline& P, SRC src, bool first, int cur, bool flat, bool
     else cudaLaunchKernelEx(&cfg, bin_kernel<SRC, false>, src, a);
 }
 
-// Enqueue n_steps steps.  dbg_for(t) gives the solve
-// kernel's optional outputs of step t; from step record_from on, a plain call
-// records the LP's active sets.
+// Enqueue n_steps steps.  dbg_for(t) gives the solve kernel's optional outputs of
+// step t; from step record_from on, a plain call records the LP's active sets.
 template <class SRC, class DBG>
 void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_delta,
                    cudaStream_t st, DBG dbg_for, int call_mode, int record_from = INT_MAX) {
@@ -543,8 +545,8 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
                                            flat || nb > 0 ? nullptr : B.key,
                                            B.slot, B.count, nullptr, nullptr};
         if (by_warp)
-            launch_warp_solve(mode, flat, by_y, wgrid, sb, st, n, src, B.pos1, B.vel1, B.aux[cur], B.start,
-                              ain, vpd, out, dbg_for(t), B.err);
+            launch_warp_solve(mode, flat, by_y, wgrid, sb, st, n, src, B.pos1, B.vel1,
+                              B.aux[cur], B.start, ain, vpd, out, dbg_for(t), B.err);
         else if (mode == MODE_RECORD)
             launch_agent_solve<SRC, MODE_RECORD>(P.kmax, P.kin, early, sgrid, sb, st, n, src, B.pos1,
                                                  B.vel1, B.aux[cur], B.start, ain, vpd, out,

@@ -45,7 +45,7 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     const int r = (int)blockIdx.x, nb = (int)gridDim.x, tid = (int)threadIdx.x;
     const int cn = 1 << sh.cell_shift, sn = 1 << sh.slot_shift;
     uint4* slots = cluster_mem;                                    // sn cell-order records
-    uint32_t* cells = reinterpret_cast<uint32_t*>(slots + sn);     // cn counts, then starts, + total
+    uint32_t* cells = reinterpret_cast<uint32_t*>(slots + sn);     // cn counts, later starts
 
     // the solve kernel may be set up meanwhile; what ran before is finished
     // before any state is read

@@ -14,9 +14,12 @@
 // exclusive scan of the cell counts, the scatter into cell order and the
 // ordering by x inside every cell) ->
 // solve (one thread per agent, or in small scenes one warp: k-nearest search
-// over the x-sorted grid rows, ORCA lines, LP, integrate) writing pos0/vel0 in sorted order, which becomes the state
-// order of the next step; the last step of a call writes the caller's
-// arrays instead.
+// over the x-sorted grid rows, ORCA lines, LP, integrate) writing pos0/vel0 in
+// sorted order, which becomes the state order of the next step; the last step
+// of a call writes the caller's arrays instead.  Scenes of up to 20,480 agents
+// are binned by one cluster in shared memory, which needs no counts from the
+// previous solve; single scenes of up to 1,024 agents have no cells: one run
+// sorted along one side of the scene's box.
 #pragma once
 
 #include <climits>

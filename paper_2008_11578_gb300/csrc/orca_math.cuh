@@ -219,10 +219,10 @@ __host__ __device__ __forceinline__ bool act_overlap(uint32_t a, int m) {
 // Velocity LP (paper Sec. 3, LP paragraphs).  Lines live in shared memory at
 // L[i * stride].  Interval bounds divide by determinants of unit directions
 // (|den| <= 2), so the fast 2-ulp division is safe and costs two
-// instructions instead of the IEEE sequence.  The objective is the Euclidean distance to v_pref, so the
-// incremental scheme is exact: when the current optimum violates line i, the
-// new optimum lies on line i, and a 1D problem on that line with the earlier
-// lines and the speed disc finds it.
+// instructions instead of the IEEE sequence.  The objective is the Euclidean
+// distance to v_pref, so the incremental scheme is exact: when the current
+// optimum violates line i, the new optimum lies on line i, and a 1D problem on
+// that line with the earlier lines and the speed disc finds it.
 // ---------------------------------------------------------------------------
 
 // Rounding allowance of the LP's emptiness tests, in m/s.  Intervals whose
@@ -756,6 +756,21 @@ __device__ __forceinline__ int solve_velocity_work_units(const float4* __restric
     return 1;
 }
 
+// The bisector of two lines as the comparison schemes build it (rounding left
+// to the compiler's contraction).
+__device__ __forceinline__ bool plain_bisector(float4 li, float4 lj, float4& b) {
+    const float ax = li.w - lj.w;
+    const float ay = lj.z - li.z;
+    const float a2 = ax * ax + ay * ay;
+    if (a2 <= 1e-12f) return false;
+    const float ci = li.z * li.y - li.w * li.x;
+    const float cj = lj.z * lj.y - lj.w * lj.x;
+    const float s = __fdividef(cj - ci, a2);
+    const float inv = rsqrtf(a2);
+    b = make_float4(ax * s, ay * s, ay * inv, -ax * inv);
+    return true;
+}
+
 // ---------------------------------------------------------------------------
 // Active-set enumeration, for comparison: every point where the optimum can
 // sit is built and tested against all half-planes and the speed disc, in an
@@ -775,21 +790,6 @@ __device__ __forceinline__ int solve_velocity_work_units(const float4* __restric
 //   valley tie-break.
 // O(k^3) work per agent, against O(k^2) for the incremental scheme.
 // ---------------------------------------------------------------------------
-// The bisector of two lines as the comparison schemes build it (rounding left
-// to the compiler's contraction).
-__device__ __forceinline__ bool plain_bisector(float4 li, float4 lj, float4& b) {
-    const float ax = li.w - lj.w;
-    const float ay = lj.z - li.z;
-    const float a2 = ax * ax + ay * ay;
-    if (a2 <= 1e-12f) return false;
-    const float ci = li.z * li.y - li.w * li.x;
-    const float cj = lj.z * lj.y - lj.w * lj.x;
-    const float s = __fdividef(cj - ci, a2);
-    const float inv = rsqrtf(a2);
-    b = make_float4(ax * s, ay * s, ay * inv, -ax * inv);
-    return true;
-}
-
 __device__ __forceinline__ float max_penetration(const float4* __restrict__ L, int stride, int n,
                                                  float x, float y) {
     float t = -CUDART_INF_F;

@@ -8,11 +8,11 @@
 //   LP           a sub-problem's bounds one per lane, merged by redux; the
 //                next violated line is found by a vote, not by a loop
 // Every expression and every discrete choice is the per-thread kernel's
-// (solve_kernel), so a step's results do not depend on which one ran.
+// (agent_solve_kernel), so a step's results do not depend on which one ran.
 // Bound by the latency of one agent's chain while the scene is small (1,000
 // agents: 51 -> 14 us a launch, about 12,500 cycles an agent: loads 1,600,
 // seed 2,100, scan 1,900, half-planes 1,400, order 900, LP 3,600), then by
-// issue slots (16,000 agents: 51 -> 40 us, 73 % of issue slots busy; eight
+// issue slots (16,000 agents: 51 -> 39.5 us, 73 % of issue slots busy; eight
 // blocks an SM 39.7 us, seven 40.9, six 41.0, five 43.0).
 #pragma once
 
@@ -243,8 +243,9 @@ __device__ __forceinline__ int warp_solve_velocity(const float4* L, float4 lj, i
 // while the ones before are tested.
 template <class SRC, int MODE, bool FLAT>
 __global__ void __launch_bounds__(128, 8)
-warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos, const float2* __restrict__ vel,
-                  const uint2* __restrict__ aux, const uint32_t* __restrict__ cstart, AgentIn ain,
+warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos,
+                  const float2* __restrict__ vel, const uint2* __restrict__ aux,
+                  const uint32_t* __restrict__ cstart, AgentIn ain,
                   const float2* __restrict__ vpd, StepOut out, DebugOut dbg,
                   int* __restrict__ err) {
     __shared__ WarpSlots slots[4];
