@@ -1090,17 +1090,19 @@ int orca_scene_remove_arrived(orca_scene* s, int* n_kept, int32_t* kept_index, v
     compact_gather_kernel<<<gb, tb, 0, st>>>(
         n, range, B.bsum, (const float2*)A.pos, (const float2*)A.vel, (const float2*)A.goal,
         A.radius, A.max_speed, A.type, A.route, (const float2*)A.waypoints, A.n_waypoints,
-        A.wp_idx, B.pos0, B.vel0, B.pos1, B.vel1, B.aux[0], B.aux[1], total);
+        A.wp_idx, B.pos0, B.vel0, B.pos1, B.vel1, B.aux[0], B.aux[1], total, kept_index);
     uint32_t kept = 0;
     if (cudaMemcpyAsync(&kept, total, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return ORCA_ERR_CUDA;
-    compact_scatter_kernel<<<std::max(1, ((int)kept + tb - 1) / tb), tb, 0, st>>>(
-        (int)kept, B.pos0, B.vel0, B.pos1, B.vel1, B.aux[0], B.aux[1], (float2*)A.pos,
-        (float2*)A.vel, (float2*)A.goal, (float*)A.radius, (float*)A.max_speed, (uint8_t*)A.type,
-        (int32_t*)A.route, A.wp_idx, kept_index, (int)kept < n ? B.err + 1 : nullptr);
-    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
-        return ORCA_ERR_CUDA;
+    if ((int)kept < n) {   // (nobody left: nothing moves)
+        compact_scatter_kernel<<<std::max(1, ((int)kept + tb - 1) / tb), tb, 0, st>>>(
+            (int)kept, B.pos0, B.vel0, B.pos1, B.vel1, B.aux[0], B.aux[1], (float2*)A.pos,
+            (float2*)A.vel, (float2*)A.goal, (float*)A.radius, (float*)A.max_speed,
+            (uint8_t*)A.type, (int32_t*)A.route, A.wp_idx, kept_index, B.err + 1);
+        if (cudaStreamSynchronize(st) != cudaSuccess) return ORCA_ERR_CUDA;
+    }
+    if (cudaGetLastError() != cudaSuccess) return ORCA_ERR_CUDA;
     P.n = (int)kept;
     drop_graph(P);   // a graph recorded for the old count is stale
     s->adj_steps = -1;
