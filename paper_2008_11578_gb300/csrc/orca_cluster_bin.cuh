@@ -35,6 +35,20 @@ inline size_t cluster_smem(ClusterShape sh) {
     return ((size_t)16 << sh.slot_shift) + ((size_t)4 << sh.cell_shift) + 16;
 }
 
+// The cluster barrier in two halves: what a block writes between them need not
+// be visible to the others, so the barrier does not wait for it, and loads that
+// need nothing from the others overlap it.  An arrival also waits until the
+// block's earlier writes have reached memory (a fence: a quarter of the kernel's
+// stalls with whole barriers), so global writes stand behind it.  1.1 us a step
+// (4,064 agents, 16 steps and their gradient 676 -> 650 us; 16,250 agents, 4 steps
+// 193 -> 189).  Every thread of every block calls both.
+__device__ __forceinline__ void cluster_arrive() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
 template <class SRC, bool FIRST>
 __global__ void __launch_bounds__(kClusterThreads)
 cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
@@ -50,6 +64,8 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     // the solve kernel may be set up meanwhile; what ran before is finished
     // before any state is read
     launch_dependents();
+    for (int q = tid; q <= cn; q += kClusterThreads) cells[q] = 0u;
+    cluster_arrive();
     wait_for_primary();
 
     // ---- the agents of this block and their cells ----
@@ -91,9 +107,8 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
         }
     }
     if (lost) atomicOr(a.err, ERR_BIT_STATE);
-    for (int q = tid; q <= cn; q += kClusterThreads) cells[q] = 0u;
     if (bad) atomicOr(a.err, ERR_BIT_NONFINITE);
-    cl.sync();
+    cluster_wait();   // every block's counts are zero
 
     // ---- counting ----
     uint32_t slot[kClusterPerThread];
@@ -105,7 +120,8 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
             slot[u] = atomicAdd(rc + (c[u] & (uint32_t)(cn - 1)), 1u);
         }
     }
-    cl.sync();
+    cluster_arrive();
+    cluster_wait();
 
     // ---- starts within the block's cells, and the blocks' totals ----
     {
@@ -126,7 +142,8 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
             total = carry;
         }
     }
-    cl.sync();
+    cluster_arrive();
+    cluster_wait();
     if (tid < 32) {
         uint32_t t = tid < nb ? *cl.map_shared_rank(&total, (unsigned)tid) : 0u;
 #pragma unroll
@@ -150,22 +167,29 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
             rs[d & (uint32_t)(sn - 1)] = make_uint4(x_order_key(x[u]), (uint32_t)from[u], b, e);
         }
     }
+    cluster_arrive();
     const int c0 = r << sh.cell_shift;
     for (int q = tid; q < cn && c0 + q < a.ncells; q += kClusterThreads)
         a.start[c0 + q] = base[r] + cells[q];
     if (r == nb - 1 && tid == 0) a.start[a.ncells] = (uint32_t)a.n;
-    cl.sync();
+    cluster_wait();
 
     // ---- order by x inside every cell (ties by slot); move the state ----
+    float2 p[kClusterPerThread], v[kClusterPerThread];
+    uint2 ax[kClusterPerThread];
+    uint32_t dst[kClusterPerThread];
 #pragma unroll
     for (int u = 0; u < kClusterPerThread; ++u) {
         const int t = i0 + tid + u * kClusterThreads;
+        p[u] = v[u] = make_float2(0.0f, 0.0f);
+        ax[u] = make_uint2(0u, 0u);
+        dst[u] = 0u;
         if (t < iend) {
             const uint4 e = slots[t - i0];
             const uint32_t i = e.y;
-            const float2 p = FIRST ? a.upos[i] : a.pos0[i];
-            const float2 v = FIRST ? a.uvel[i] : a.vel0[i];
-            const uint2 ax = FIRST ? aux_pack(a.urad[i], a.utype[i], (int)i) : a.aux0[i];
+            p[u] = FIRST ? a.upos[i] : a.pos0[i];
+            v[u] = FIRST ? a.uvel[i] : a.vel0[i];
+            ax[u] = FIRST ? aux_pack(a.urad[i], a.utype[i], (int)i) : a.aux0[i];
             uint32_t rank = 0u;
             for (uint32_t w = e.z; w < e.w; ++w) {
                 const unsigned own = (unsigned)(w >> sh.slot_shift);
@@ -173,13 +197,19 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
                 const uint32_t xv = rs[w & (uint32_t)(sn - 1)].x;
                 rank += (xv < e.x || (xv == e.x && w < (uint32_t)t)) ? 1u : 0u;
             }
-            const uint32_t dst = e.z + rank;
-            a.pos1[dst] = p;
-            a.vel1[dst] = v;
-            a.aux1[dst] = ax;
+            dst[u] = e.z + rank;
         }
     }
-    cl.sync();   // no block leaves while another reads its records
+    cluster_arrive();
+#pragma unroll
+    for (int u = 0; u < kClusterPerThread; ++u) {
+        if (i0 + tid + u * kClusterThreads < iend) {
+            a.pos1[dst[u]] = p[u];
+            a.vel1[dst[u]] = v[u];
+            a.aux1[dst[u]] = ax[u];
+        }
+    }
+    cluster_wait();   // no block leaves while another reads its records
 }
 
 // ------------------------------------------------------- no cells at all ----
