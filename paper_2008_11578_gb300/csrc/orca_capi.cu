@@ -1261,7 +1261,7 @@ int orca_adjoint(orca_scene* s, int n_steps, int ckpt_every, const float* vpref_
                 bp[nx], bv[nx], dl_dvel_traj ? (const float2*)dl_dvel_traj + tn : nullptr,
                 bp[cu], bv[cu], bp[sp], bv[sp],
                 dl_dvpref_delta ? (float2*)dl_dvpref_delta + tn : nullptr,
-                (float2*)dl_dwaypoints, s->p.buf.err);
+                (float2*)dl_dwaypoints, s->p.buf.err, t < t1 - 1);
             const int old_nx = nx;
             nx = cu;
             cu = sp;
@@ -1328,7 +1328,7 @@ int orca_step_vjp(orca_scene* s, void* adj_ws, size_t adj_bytes, const float* po
         stm, n, s->p.one, rec.r_pos, rec.r_vel, A.radius, A.type, rec.r_nbr, rec.k, rec.r_act,
         rec.r_wp, rec.r_vnew, ain, (const float2*)vpref_delta, (const float2*)dl_dpos_next,
         (const float2*)dl_dvel_next, nullptr, bp[1], bv[1], bp[2], bv[2],
-        (float2*)dl_dvpref_delta, (float2*)dl_dwaypoints, s->p.buf.err);
+        (float2*)dl_dvpref_delta, (float2*)dl_dwaypoints, s->p.buf.err, false);
     ok = cudaMemcpyAsync(dl_dpos, bp[1], nb, cudaMemcpyDeviceToDevice, stm) == cudaSuccess &&
          cudaMemcpyAsync(dl_dvel, bv[1], nb, cudaMemcpyDeviceToDevice, stm) == cudaSuccess;
     if (!ok) return ORCA_ERR_CUDA;
