@@ -773,7 +773,8 @@ def run_ours(args):
                     "peak_warp_inst_per_s": 4.0 * sms * float(sm_mhz) * 1e6,
                     "frac": prof["warp_instructions_per_launch"] / solve_avg_s
                             / (4.0 * sms * float(sm_mhz) * 1e6)},
-                "kernel": "solve_kernel", "solve_ms": statistics.mean(solve_ms),
+                "kernel": "agent_solve_kernel (small scenes: warp_solve_kernel)",
+                "solve_ms": statistics.mean(solve_ms),
                 "solve_share_of_step": statistics.mean(solve_ms) / statistics.mean(step_ms),
                 "flops_per_agent_step": flops / n,
                 "counts_per_agent": {"candidates": c[0] / n, "neighbours": c[1] / n,
