@@ -417,11 +417,23 @@ static_assert(kClusterBinMax <= kClusterMax * kClusterSlots, "a cluster holds th
 
 // Blocks of the cluster that bins the scene (0: it takes bin_kernel instead):
 // about one agent per thread, more where the cells need the shared memory.
+// Blocks of 512 threads where 16 of them have a thread for every agent: their
+// barriers and scans are shorter (8,191 agents with k = 32, 2 steps 105 -> 102 us;
+// 4,064 agents, 16 steps and their gradient 618 -> 603); with two or more agents a
+// thread blocks of 1,024 are ahead (48 scenes, 19,000 agents, 4 steps 200 -> 196).
 int bin_cluster(const Pipeline& P, ClusterShape* sh) {
     if (P.n > kClusterBinMax || (P.flags & ORCA_DEBUG_BARRIER_TIMEOUT)) return 0;
     for (int nb = 1; nb <= P.cluster_max; nb *= 2) {
+        ClusterShape s{2, 0, kClusterThreadsFew};
+        while (((long long)nb << s.cell_shift) < P.ncells) ++s.cell_shift;
+        while (((long long)nb << s.slot_shift) < P.n) ++s.slot_shift;
+        if ((1 << s.cell_shift) > kClusterCellsFew || (1 << s.slot_shift) > s.threads) continue;
+        *sh = s;
+        return nb;
+    }
+    for (int nb = 1; nb <= P.cluster_max; nb *= 2) {
         const bool last = nb * 2 > P.cluster_max;
-        ClusterShape s{2, 0};
+        ClusterShape s{2, 0, kClusterThreads};
         while (((long long)nb << s.cell_shift) < P.ncells) ++s.cell_shift;
         while (((long long)nb << s.slot_shift) < P.n) ++s.slot_shift;
         if ((1 << s.cell_shift) > kClusterCells) continue;
@@ -460,7 +472,7 @@ void launch_bin(const Pipeline& P, SRC src, bool first, int cur, bool flat, bool
     if (nb > 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)nb);
-        cfg.blockDim = dim3(kClusterThreads);
+        cfg.blockDim = dim3((unsigned)sh.threads);
         cfg.dynamicSmemBytes = cluster_smem(sh);
         cfg.stream = st;
         cudaLaunchAttribute attr[2];
@@ -470,8 +482,13 @@ void launch_bin(const Pipeline& P, SRC src, bool first, int cur, bool flat, bool
         attr[1] = programmatic_launch();
         cfg.attrs = attr;
         cfg.numAttrs = 2;
-        if (first) cudaLaunchKernelEx(&cfg, cluster_bin_kernel<SRC, true>, src, a, sh);
-        else cudaLaunchKernelEx(&cfg, cluster_bin_kernel<SRC, false>, src, a, sh);
+        cudaLaunchKernelEx(&cfg,
+                           sh.threads == kClusterThreadsFew
+                               ? (first ? cluster_bin_kernel<SRC, true, kClusterThreadsFew>
+                                        : cluster_bin_kernel<SRC, false, kClusterThreadsFew>)
+                               : (first ? cluster_bin_kernel<SRC, true, kClusterThreads>
+                                        : cluster_bin_kernel<SRC, false, kClusterThreads>),
+                           src, a, sh);
         return;
     }
     const long long work = std::max((long long)P.n, (long long)P.ncells / 4);
@@ -507,7 +524,7 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
     const size_t smem = solve_smem(P);
     const bool by_warp = solve_by_warp(P, call_mode);
     const bool flat = solve_flat(P, by_warp), by_y = flat && flat_by_y(P);
-    ClusterShape shape{0, 0};
+    ClusterShape shape{0, 0, 0};
     const int nb = bin_cluster(P, &shape);
     // The per-thread solve kernel is set up during the binning only when its
     // blocks go over more than one wave: placed while the binning blocks still
@@ -596,7 +613,10 @@ template <class SRC>
 cudaError_t cluster_max(int* out) {
     *out = 0;
     const size_t smem = (size_t)16 * kClusterSlots + (size_t)4 * kClusterCells + 16;
-    for (auto f : {cluster_bin_kernel<SRC, true>, cluster_bin_kernel<SRC, false>}) {
+    for (auto f : {cluster_bin_kernel<SRC, true, kClusterThreads>,
+                   cluster_bin_kernel<SRC, false, kClusterThreads>,
+                   cluster_bin_kernel<SRC, true, kClusterThreadsFew>,
+                   cluster_bin_kernel<SRC, false, kClusterThreadsFew>}) {
         cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (e == cudaSuccess)
@@ -615,10 +635,10 @@ cudaError_t cluster_max(int* out) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int k0 = 0, k1 = 0;
-        if (cudaOccupancyMaxActiveClusters(&k0, cluster_bin_kernel<SRC, true>, &cfg) ==
-                cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&k1, cluster_bin_kernel<SRC, false>, &cfg) ==
-                cudaSuccess &&
+        if (cudaOccupancyMaxActiveClusters(&k0, cluster_bin_kernel<SRC, true, kClusterThreads>,
+                                           &cfg) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&k1, cluster_bin_kernel<SRC, false, kClusterThreads>,
+                                           &cfg) == cudaSuccess &&
             k0 > 0 && k1 > 0) {
             *out = nb;
             break;

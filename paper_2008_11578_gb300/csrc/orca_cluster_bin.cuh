@@ -25,10 +25,14 @@ constexpr int kClusterPerThread = 2;                                 // agents
 constexpr int kClusterSlots = kClusterThreads * kClusterPerThread;   // per block
 constexpr int kClusterCells = 32768;                                 // per block
 
-// log2 sizes of the cell and slot ranges of a block
+constexpr int kClusterThreadsFew = 512;    // threads of a block in scenes of few agents
+constexpr int kClusterCellsFew = 4096;     // and few cells
+
+// log2 sizes of the cell and slot ranges of a block, and its threads
 struct ClusterShape {
     int cell_shift;
     int slot_shift;
+    int threads;
 };
 
 inline size_t cluster_smem(ClusterShape sh) {
@@ -49,8 +53,8 @@ __device__ __forceinline__ void cluster_wait() {
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-template <class SRC, bool FIRST>
-__global__ void __launch_bounds__(kClusterThreads)
+template <class SRC, bool FIRST, int NT>
+__global__ void __launch_bounds__(NT)
 cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     namespace cg = cooperative_groups;
     extern __shared__ uint4 cluster_mem[];
@@ -64,7 +68,7 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     // the solve kernel may be set up meanwhile; what ran before is finished
     // before any state is read
     launch_dependents();
-    for (int q = tid; q <= cn; q += kClusterThreads) cells[q] = 0u;
+    for (int q = tid; q <= cn; q += NT) cells[q] = 0u;
     cluster_arrive();
     wait_for_primary();
 
@@ -81,7 +85,7 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     bool bad = false, lost = false;
 #pragma unroll
     for (int u = 0; u < kClusterPerThread; ++u) {
-        from[u] = i0 + tid + u * kClusterThreads;
+        from[u] = i0 + tid + u * NT;
         if (FIRST && hint != nullptr && from[u] < iend) {
             const uint32_t h = __ldg(hint + from[u]);
             if (h < (uint32_t)a.n) from[u] = (int)h;
@@ -92,7 +96,7 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     for (int u = 0; u < kClusterPerThread; ++u) {
         c[u] = 0xffffffffu;
         x[u] = 0.0f;
-        if (i0 + tid + u * kClusterThreads < iend) {
+        if (i0 + tid + u * NT < iend) {
             const int i = from[u];
             const float2 p = FIRST ? a.upos[i] : a.pos0[i];
             if (FIRST) {
@@ -126,7 +130,7 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     // ---- starts within the block's cells, and the blocks' totals ----
     {
         uint32_t carry = 0u;
-        for (int q0 = 0; q0 < cn; q0 += 4 * kClusterThreads) {
+        for (int q0 = 0; q0 < cn; q0 += 4 * NT) {
             const int q = q0 + 4 * tid;
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
             if (q < cn) v = *reinterpret_cast<const uint4*>(cells + q);
@@ -169,7 +173,7 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     }
     cluster_arrive();
     const int c0 = r << sh.cell_shift;
-    for (int q = tid; q < cn && c0 + q < a.ncells; q += kClusterThreads)
+    for (int q = tid; q < cn && c0 + q < a.ncells; q += NT)
         a.start[c0 + q] = base[r] + cells[q];
     if (r == nb - 1 && tid == 0) a.start[a.ncells] = (uint32_t)a.n;
     cluster_wait();
@@ -180,7 +184,7 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     uint32_t dst[kClusterPerThread];
 #pragma unroll
     for (int u = 0; u < kClusterPerThread; ++u) {
-        const int t = i0 + tid + u * kClusterThreads;
+        const int t = i0 + tid + u * NT;
         p[u] = v[u] = make_float2(0.0f, 0.0f);
         ax[u] = make_uint2(0u, 0u);
         dst[u] = 0u;
@@ -203,7 +207,7 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     cluster_arrive();
 #pragma unroll
     for (int u = 0; u < kClusterPerThread; ++u) {
-        if (i0 + tid + u * kClusterThreads < iend) {
+        if (i0 + tid + u * NT < iend) {
             a.pos1[dst[u]] = p[u];
             a.vel1[dst[u]] = v[u];
             a.aux1[dst[u]] = ax[u];

@@ -39,6 +39,13 @@ def test_slot_ranges(n):
     _check(scenes.open_square(n, (n / 0.4) ** 0.5 + 1.0, seed=91))
 
 
+@pytest.mark.parametrize("n, cell", [(512, None), (513, None), (8192, None), (8193, None),
+                                     (2000, 1.1), (2000, 1.05), (8192, 0.55)])
+def test_block_sizes(n, cell):
+    """One agent and more per thread, few and many cells per block."""
+    _check(scenes.open_square(n, (n / 0.4) ** 0.5 + 1.0, seed=95), cell)
+
+
 @pytest.mark.parametrize("cell", [0.19, 0.08, 400.0])
 def test_cell_ranges(cell):
     """69k cells (more blocks than the agents need), 391k cells, one cell."""
