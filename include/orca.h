@@ -348,8 +348,7 @@ int orca_adjoint_workspace_bytes(const orca_scene *scene, int n_steps, int ckpt_
                                  size_t *out_bytes);
 
 /*
- * orca_step over n_steps steps that also stores checkpoints and, for the
- * adjoint, the records of the last ckpt_every-step segment in adj_ws
+ * orca_step over n_steps steps that also stores checkpoints in adj_ws
  * (device, 256-byte aligned, orca_adjoint_workspace_bytes bytes) and, when
  * vel_traj != NULL, writes the velocity after every step into vel_traj
  * (float2[n_steps * N], step-major, caller order).  The scene's pos, vel and
@@ -394,9 +393,7 @@ int orca_step_vjp(orca_scene *scene, void *adj_ws, size_t adj_bytes, const float
                   const float *dl_dpos_next, const float *dl_dvel_next, float *dl_dpos,
                   float *dl_dvel, float *dl_dvpref_delta, float *dl_dwaypoints, void *stream);
 
-/* Kernel launches of one orca_adjoint call at most (replays and adjoint
-   kernels); the first call after an orca_rollout, neither of them in a stream
-   capture, saves the last segment's replay, which the rollout recorded. */
+/* Kernel launches of one orca_adjoint call (replays and adjoint kernels). */
 int orca_adjoint_launch_count(const orca_scene *scene, int n_steps, int ckpt_every);
 
 /*

@@ -290,7 +290,7 @@ adjoint_kernel(int n, SceneDev sc, const float2* __restrict__ pos, const float2*
     // lane m's active line, rebuilt from the recorded state
     const uint32_t ac = act[A];
     const int nl = act_nlines(ac);
-    bool line = q < nl;   // (at most three)
+    const bool line = q < nl;   // (at most three)
     const float2 p = pos[A], v = vel[A];
     const float r = rad[A];
     const int ta = typ[A];
@@ -298,12 +298,8 @@ adjoint_kernel(int n, SceneDev sc, const float2* __restrict__ pos, const float2*
     float2 pj = p, vj = v;
     float rj = 0.0f, f = 0.0f;
     float4 mine = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (line) {   // (no index of a record that is none is followed)
-        j = nbr[(size_t)A * k_stride + min(act_line(ac, q), k_stride - 1)];
-        line = j >= 0 && j < n;
-        if (!line) j = A;
-    }
     if (line) {
+        j = nbr[(size_t)A * k_stride + act_line(ac, q)];
         pj = pos[j];
         vj = vel[j];
         rj = rad[j];
@@ -328,7 +324,7 @@ adjoint_kernel(int n, SceneDev sc, const float2* __restrict__ pos, const float2*
     if (ain.route != nullptr) {
         rt = ain.route[A];
         if (rt >= 0) {
-            wi = min((int)wp_used[A], ain.n_waypoints - 1);
+            wi = wp_used[A];
             g = ain.waypoints[(size_t)rt * ain.n_waypoints + wi];
         }
     }

@@ -509,10 +509,10 @@ void launch_bin(const Pipeline& P, SRC src, bool first, int cur, bool flat, bool
 }
 
 // Enqueue n_steps steps.  dbg_for(t) gives the solve kernel's optional outputs of
-// step t; from step record_from on, a plain call records the LP's active sets.
+// step t.
 template <class SRC, class DBG>
 void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_delta,
-                   cudaStream_t st, DBG dbg_for, int call_mode, int record_from = INT_MAX) {
+                   cudaStream_t st, DBG dbg_for, int mode) {
     const int n = P.n;
     const Buffers& B = P.buf;
     const orca_agents& A = P.agents;
@@ -522,7 +522,7 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
     int sb = P.block;
     int sgrid = (n + sb - 1) / sb;
     const size_t smem = solve_smem(P);
-    const bool by_warp = solve_by_warp(P, call_mode);
+    const bool by_warp = solve_by_warp(P, mode);
     const bool flat = solve_flat(P, by_warp), by_y = flat && flat_by_y(P);
     ClusterShape shape{0, 0, 0};
     const int nb = bin_cluster(P, &shape);
@@ -534,7 +534,7 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
     const bool early = sgrid > 2 * P.bin_grid_max;
     // Grids of several waves end more evenly in blocks of two warps, unless the
     // caller chose the size (1M clusters 375 -> 367 us, 250,000 138 -> 136).
-    if (P.any_block && early && (call_mode == MODE_PLAIN || call_mode == MODE_RECORD)) {
+    if (P.any_block && early && (mode == MODE_PLAIN || mode == MODE_RECORD)) {
         sb = 64;
         sgrid = (n + sb - 1) / sb;
     }
@@ -555,7 +555,6 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
             vpref_delta ? (const float2*)vpref_delta + (size_t)t * (size_t)n : nullptr;
         if (P.ev_begin) cudaEventRecord(P.ev_begin, st);
         const bool last = t == n_steps - 1;
-        const int mode = t >= record_from ? MODE_RECORD : call_mode;
         const StepOut out = last ? StepOut{(float2*)A.pos, (float2*)A.vel, true, nullptr, nullptr,
                                            nullptr, B.hint, B.err + 1}
                                  : StepOut{B.pos0, B.vel0, false,
@@ -845,8 +844,6 @@ struct orca_scene {
     int adj_steps;
     int adj_every;
     void* adj_ws;
-    // the segment whose records adj_ws holds for the adjoint (-1: none)
-    int adj_recorded;
 };
 
 namespace {
@@ -908,35 +905,6 @@ struct ReplayDebug {
         return d;
     }
 };
-
-ReplayDebug replay_debug(char* w, const AdjLayout& L, bool routed, int n, int k) {
-    ReplayDebug r{DebugOut{}, (float2*)(w + L.r_pos), (float2*)(w + L.r_vel),
-                  (int32_t*)(w + L.r_nbr), (uint32_t*)(w + L.r_act),
-                  routed ? (uint8_t*)(w + L.r_wp) : nullptr, (float2*)(w + L.r_vnew), n,
-                  std::max(k, 1)};
-    r.base.k_stride = std::max(k, 1);
-    return r;
-}
-
-// Outputs of a rollout that records its last segment (steps from record_from
-// on) for the adjoint.
-struct RecordingDebug {
-    RolloutDebug rollout;
-    ReplayDebug replay;
-    int record_from;
-    __host__ DebugOut operator()(int t) const {
-        const DebugOut d = rollout(t);
-        if (t < record_from) return d;
-        DebugOut r = replay(t - record_from);
-        r.swp = d.swp;
-        return r;
-    }
-};
-
-bool capturing(cudaStream_t st) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
-}
 
 // The adjoint kernel of one step: four lanes per agent.
 template <class... ARGS>
@@ -1008,7 +976,6 @@ int orca_scene_create(const orca_params* params, const orca_agents* agents, void
     s->adj_steps = -1;
     s->adj_every = 0;
     s->adj_ws = nullptr;
-    s->adj_recorded = -1;
     // the binning kernel expects zero cell counts on entry
     if (cudaMemset(s->p.buf.err, 0, 16) != cudaSuccess ||
         cudaMemset(s->p.buf.count, 0, ncells * 4) != cudaSuccess || prepare(s->p) != ORCA_OK) {
@@ -1075,9 +1042,7 @@ int orca_scene_graph_launch(orca_scene* s, void* stream) {
 
 int orca_scene_sync_status(orca_scene* s) {
     if (!s) return ORCA_ERR_INVALID_ARG;
-    const int st = read_status(s->p);
-    if (st != ORCA_OK) s->adj_recorded = -1;   // a step that gave up recorded nothing
-    return st;
+    return read_status(s->p);
 }
 
 void orca_scene_destroy(orca_scene* s) {
@@ -1126,7 +1091,6 @@ int orca_scene_remove_arrived(orca_scene* s, int* n_kept, int32_t* kept_index, v
     P.n = (int)kept;
     drop_graph(P);   // a graph recorded for the old count is stale
     s->adj_steps = -1;
-    s->adj_recorded = -1;
     *n_kept = (int)kept;
     return ORCA_OK;
 }
@@ -1153,7 +1117,6 @@ int orca_rollout(orca_scene* s, int n_steps, int ckpt_every, const float* vpref_
     if (st != ORCA_OK) return st;
     if (vel_traj && !aligned(vel_traj, 8)) return ORCA_ERR_INVALID_ARG;
     s->adj_steps = -1;
-    s->adj_recorded = -1;
     const int n = s->p.n;
     if (n > 0 && n_steps > 0) {
         const AdjLayout L = make_adj_layout((size_t)n, s->params.max_neighbors, n_steps,
@@ -1163,34 +1126,10 @@ int orca_rollout(orca_scene* s, int n_steps, int ckpt_every, const float* vpref_
                          (float2*)(w + L.ck_vel),
                          s->p.agents.route ? (uint8_t*)(w + L.ck_wp) : nullptr, n, ckpt_every};
         dbg.base.k_stride = s->params.max_neighbors;
-        cudaStream_t stm = (cudaStream_t)stream;
-        // The adjoint starts with the last segment: its records are written
-        // here, as its replay would write them, and the checkpoint and the
-        // velocities copied out of them, so that the adjoint need not replay it
-        // (not into a graph, whose adjoint may run more than once per rollout).
-        const bool record = !capturing(stm);
-        const int t_rec = (L.n_ck - 1) * ckpt_every;
-        if (record) {
-            const ReplayDebug rec = replay_debug(w, L, s->p.agents.route != nullptr, n,
-                                                 s->params.max_neighbors);
-            enqueue_steps(s->p, OneScene{s->p.one}, n_steps, vpref_delta, stm,
-                          RecordingDebug{dbg, rec, t_rec}, MODE_PLAIN, t_rec);
-            const size_t nb = (size_t)n * 8, c = (size_t)(L.n_ck - 1) * n;
-            if (cudaMemcpyAsync(dbg.ck_pos + c, rec.r_pos, nb, cudaMemcpyDeviceToDevice, stm) !=
-                    cudaSuccess ||
-                cudaMemcpyAsync(dbg.ck_vel + c, rec.r_vel, nb, cudaMemcpyDeviceToDevice, stm) !=
-                    cudaSuccess ||
-                (vel_traj &&
-                 cudaMemcpyAsync((float2*)vel_traj + (size_t)t_rec * n, rec.r_vnew,
-                                 nb * (size_t)(n_steps - t_rec), cudaMemcpyDeviceToDevice, stm) !=
-                     cudaSuccess))
-                return ORCA_ERR_CUDA;
-        } else {
-            enqueue_steps(s->p, OneScene{s->p.one}, n_steps, vpref_delta, stm, dbg, MODE_PLAIN);
-        }
+        enqueue_steps(s->p, OneScene{s->p.one}, n_steps, vpref_delta, (cudaStream_t)stream, dbg,
+                      MODE_PLAIN);
         st = cuda_status(cudaGetLastError());
         if (st != ORCA_OK) return st;
-        s->adj_recorded = record ? L.n_ck - 1 : -1;
     }
     s->adj_steps = n_steps;
     s->adj_every = ckpt_every;
@@ -1248,28 +1187,27 @@ int orca_adjoint(orca_scene* s, int n_steps, int ckpt_every, const float* vpref_
     R.ev_begin = R.ev_end = R.bin_begin = R.bin_end = nullptr;
     R.counters = nullptr;
     R.graph = nullptr;
-    const ReplayDebug rec = replay_debug(w, L, A.route != nullptr, n, k);
+    ReplayDebug rec{DebugOut{}, (float2*)(w + L.r_pos), (float2*)(w + L.r_vel),
+                    (int32_t*)(w + L.r_nbr), (uint32_t*)(w + L.r_act),
+                    A.route ? (uint8_t*)(w + L.r_wp) : nullptr, (float2*)(w + L.r_vnew), n,
+                    std::max(k, 1)};
+    rec.base.k_stride = std::max(k, 1);
     const AgentIn ain{(const float2*)A.goal, A.max_speed, A.route, (const float2*)A.waypoints,
                       A.n_waypoints, A.wp_idx};
     int nx = 0, cu = 1, sp = 2;
-    // the segment that need not be replayed; afterwards adj_ws holds the first's
-    const int recorded = capturing(stm) ? -1 : s->adj_recorded;
-    s->adj_recorded = L.n_ck == 1 ? recorded : -1;
     for (int seg = L.n_ck - 1; seg >= 0; --seg) {
         const int t0 = seg * ckpt_every;
         const int t1 = std::min(n_steps, t0 + ckpt_every);
-        if (seg != recorded) {
-            const size_t c = (size_t)seg * n;
-            ok = cudaMemcpyAsync(R.agents.pos, (float2*)(w + L.ck_pos) + c, nb,
-                                 cudaMemcpyDeviceToDevice, stm) == cudaSuccess &&
-                 cudaMemcpyAsync(R.agents.vel, (float2*)(w + L.ck_vel) + c, nb,
-                                 cudaMemcpyDeviceToDevice, stm) == cudaSuccess &&
-                 (!A.route || cudaMemcpyAsync(R.agents.wp_idx, (uint8_t*)(w + L.ck_wp) + c, n,
-                                              cudaMemcpyDeviceToDevice, stm) == cudaSuccess);
-            if (!ok) return ORCA_ERR_CUDA;
-            const float* vpd0 = vpref_delta ? vpref_delta + (size_t)t0 * n * 2 : nullptr;
-            enqueue_steps(R, OneScene{R.one}, t1 - t0, vpd0, stm, rec, MODE_RECORD);
-        }
+        const size_t c = (size_t)seg * n;
+        ok = cudaMemcpyAsync(R.agents.pos, (float2*)(w + L.ck_pos) + c, nb,
+                             cudaMemcpyDeviceToDevice, stm) == cudaSuccess &&
+             cudaMemcpyAsync(R.agents.vel, (float2*)(w + L.ck_vel) + c, nb,
+                             cudaMemcpyDeviceToDevice, stm) == cudaSuccess &&
+             (!A.route || cudaMemcpyAsync(R.agents.wp_idx, (uint8_t*)(w + L.ck_wp) + c, n,
+                                          cudaMemcpyDeviceToDevice, stm) == cudaSuccess);
+        if (!ok) return ORCA_ERR_CUDA;
+        const float* vpd0 = vpref_delta ? vpref_delta + (size_t)t0 * n * 2 : nullptr;
+        enqueue_steps(R, OneScene{R.one}, t1 - t0, vpd0, stm, rec, MODE_RECORD);
         for (int t = t1 - 1; t >= t0; --t) {
             const size_t o = (size_t)(t - t0) * n;
             const size_t tn = (size_t)t * n;
@@ -1314,7 +1252,6 @@ int orca_step_vjp(orca_scene* s, void* adj_ws, size_t adj_bytes, const float* po
         return ORCA_ERR_INVALID_ARG;
     if ((A.route != nullptr) != (wp_idx != nullptr)) return ORCA_ERR_INVALID_ARG;
     if (dl_dwaypoints && !A.route) return ORCA_ERR_INVALID_ARG;
-    if (adj_ws == s->adj_ws) s->adj_recorded = -1;   // overwritten below
     cudaStream_t stm = (cudaStream_t)stream;
     const int k = s->params.max_neighbors;
     const AdjLayout L = make_adj_layout((size_t)n, k, 1, 1);
@@ -1340,7 +1277,11 @@ int orca_step_vjp(orca_scene* s, void* adj_ws, size_t adj_bytes, const float* po
     ok = ok && cudaMemsetAsync(bp[1], 0, nb, stm) == cudaSuccess &&
          cudaMemsetAsync(bv[1], 0, nb, stm) == cudaSuccess;
     if (!ok) return ORCA_ERR_CUDA;
-    const ReplayDebug rec = replay_debug(w, L, A.route != nullptr, n, k);
+    ReplayDebug rec{DebugOut{}, (float2*)(w + L.r_pos), (float2*)(w + L.r_vel),
+                    (int32_t*)(w + L.r_nbr), (uint32_t*)(w + L.r_act),
+                    A.route ? (uint8_t*)(w + L.r_wp) : nullptr, (float2*)(w + L.r_vnew), n,
+                    std::max(k, 1)};
+    rec.base.k_stride = std::max(k, 1);
     enqueue_steps(R, OneScene{R.one}, 1, vpref_delta, stm, rec, MODE_RECORD);
     const AgentIn ain{(const float2*)A.goal, A.max_speed, A.route, (const float2*)A.waypoints,
                       A.n_waypoints, A.wp_idx};
