@@ -283,7 +283,7 @@ adjoint_kernel(int n, SceneDev sc, const float2* __restrict__ pos, const float2*
         wait_for_primary();
         return;
     }
-    const int a_raw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 2);
+    const int a_raw = lane_group(blockIdx.x, blockDim.x, threadIdx.x, 4u);
     const int q = threadIdx.x & 3;
     const bool on = a_raw < n;
     const int A = on ? a_raw : n - 1;   // lanes past the end shadow the last agent, writing nothing

@@ -49,6 +49,14 @@ struct SceneDev {
     float accel_dt;             // largest forward speed gain per step
 };
 
+// The agent of a thread where `lanes` consecutive threads share one.  (Not
+// (block * threads + thread) / lanes: that product wraps at 2^32 threads, which is
+// 2^27 agents with a warp each.)
+__host__ __device__ __forceinline__ int lane_group(unsigned block, unsigned threads,
+                                                   unsigned thread, unsigned lanes) {
+    return (int)(block * (threads / lanes) + thread / lanes);
+}
+
 // kinematic half-planes a vehicle can add to its LP
 constexpr int kKinLines = 3;
 

@@ -251,7 +251,7 @@ warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos,
     __shared__ WarpSlots slots[4];
     const int lane = threadIdx.x & 31;
     WarpSlots& W = slots[threadIdx.x >> 5];
-    const int s = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int s = lane_group(blockIdx.x, blockDim.x, threadIdx.x, 32u);
     launch_dependents();
     wait_for_primary();
     if (s >= n) return;
