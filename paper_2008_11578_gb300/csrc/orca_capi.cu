@@ -37,6 +37,7 @@ using namespace orca;
 namespace {
 
 constexpr size_t kAlign = 256;
+constexpr int kMaxBlock = 128;   // threads of a solve block at most
 static_assert(kRemoveBlocks <= kBinGridMax, "the removal's block sums fit the binning's");
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -134,7 +135,8 @@ int check_params(const orca_params* p) {
     if (p->grid_nx < 1 || p->grid_ny < 1) return ORCA_ERR_INVALID_ARG;
     if ((long long)p->grid_nx * (long long)p->grid_ny > (long long)ORCA_MAX_CELLS)
         return ORCA_ERR_CAPACITY;
-    if (p->block_size != 0 && (p->block_size < 32 || p->block_size > 128 || p->block_size % 32))
+    if (p->block_size != 0 &&
+        (p->block_size < 32 || p->block_size > kMaxBlock || p->block_size % 32))
         return ORCA_ERR_INVALID_ARG;
     const unsigned schemes = ORCA_FLAG_LP_WORK_UNITS | ORCA_FLAG_LP_ENUMERATION |
                              ORCA_FLAG_LP_WARP | ORCA_DEBUG_CHECKED;
@@ -218,6 +220,7 @@ int cuda_status(cudaError_t e) { return e == cudaSuccess ? ORCA_OK : ORCA_ERR_CU
 // float4 slots per thread: the neighbour list, then the lines (plus the
 // vehicles' kinematic half-planes)
 int kcap_for(int k, bool kin) { return std::max(k, 1) + (kin ? kKinLines : 0); }
+size_t lines_smem(int kcap, int block) { return (size_t)kcap * block * sizeof(float4); }
 bool kinematic(const orca_params* p) {
     return p->vehicle_turn_rate > 0.0f || p->vehicle_accel > 0.0f;
 }
@@ -231,25 +234,29 @@ size_t agent_smem(int k, bool kin, int block) {
     return (size_t)agent_units(kl) * block * sizeof(float4);
 }
 
-// More than 48 KB of dynamic shared memory needs an explicit opt-in, set
-// once per scene/batch on its device (outside any stream capture).
+// More than 48 KB of dynamic shared memory needs an explicit opt-in, set when a
+// scene or batch that needs it is made (outside any stream capture).  It belongs
+// to the kernel, not to the scene, so it is the most that any scene takes: a
+// scene made later must not lower it for one made before.
 template <class K>
-void allow_smem(cudaError_t& e, K kernel, size_t smem) {
+void allow_smem(cudaError_t& e, K kernel, size_t smem, size_t most) {
     if (e == cudaSuccess && smem > 48 * 1024)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
 template <class SRC>
 cudaError_t prepare_solve(size_t smem, size_t smem_agent) {
+    const size_t most = lines_smem(kcap_for(ORCA_MAX_NEIGHBORS, true), kMaxBlock);
+    const size_t most_agent = agent_smem(ORCA_MAX_NEIGHBORS, true, kMaxBlock);
     cudaError_t e = cudaSuccess;
-    allow_smem(e, solve_kernel<SRC, MODE_COUNT, LP_INCREMENTAL>, smem);
-    allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_WORK_UNITS>, smem);
-    allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_ENUMERATION>, smem);
-    allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_WARP>, smem);
-    allow_smem(e, solve_kernel<SRC, MODE_CHECK, LP_INCREMENTAL>, smem);
+    allow_smem(e, solve_kernel<SRC, MODE_COUNT, LP_INCREMENTAL>, smem, most);
+    allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_WORK_UNITS>, smem, most);
+    allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_ENUMERATION>, smem, most);
+    allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_WARP>, smem, most);
+    allow_smem(e, solve_kernel<SRC, MODE_CHECK, LP_INCREMENTAL>, smem, most);
     // (10 and 16 neighbour slots stay below 48 KB)
-    allow_smem(e, agent_solve_kernel<SRC, MODE_PLAIN, 32>, smem_agent);
-    allow_smem(e, agent_solve_kernel<SRC, MODE_RECORD, 32>, smem_agent);
+    allow_smem(e, agent_solve_kernel<SRC, MODE_PLAIN, 32>, smem_agent, most_agent);
+    allow_smem(e, agent_solve_kernel<SRC, MODE_RECORD, 32>, smem_agent, most_agent);
     return e;
 }
 
@@ -358,7 +365,7 @@ struct Pipeline {
     int cluster_max;    // blocks of the largest cluster that runs here (small scenes)
 };
 
-size_t solve_smem(const Pipeline& P) { return (size_t)P.kcap * P.block * sizeof(float4); }
+size_t solve_smem(const Pipeline& P) { return lines_smem(P.kcap, P.block); }
 
 // The solve variant and diagnostics of an ordinary step.
 struct SameDebug {
