@@ -5,8 +5,13 @@
 // whatever their candidates are).  An entry is the distance d^2 with its lowest
 // bits replaced by the candidate's place in a list of admitted slots in shared
 // memory, so the order of the neighbours falls out of the network.  Where two
-// distances differ only in the replaced bits (some 5e-4 of the agents, or
-// lattices) the list is put in order exactly.
+// distances differ only in the replaced bits (some 5e-4 of the agents, or every
+// one on a regular grid) the run of them is put in order exactly (order_ties):
+// 1M agents on a grid of 1 m 392 -> 238 us against an ordering of the whole list by
+// all pairs (186 with a sorted list in shared memory), and, as one agent in a warp
+// is enough to make it wait, 53 -> 47 us for the 65,000-agent shared space.  An
+// agent with more candidates at nearly one distance than the list holds searches
+// again with a sorted list (sorted_search): 40,000 agents at 40 points 64 -> 0.9 ms.
 //
 // Bound by issue slots in large scenes (0.74 of one instruction a cycle per
 // scheduler, 57 % of an instruction's lanes active: the LP's re-solves and the
@@ -48,6 +53,154 @@ __device__ __forceinline__ void insert_pair(float (&D)[N], float a, float b) {
 // words (the neighbours in order, then each line's penetration at v_A).  The
 // search's list of admitted slots lives in the line slots.
 __host__ __device__ constexpr int agent_units(int kl) { return kl + (kl + 3) / 4; }
+
+// The two rare paths of the search, kept small (no unrolling, the second out of
+// line): with them unrolled in place 1M clusters took 380-455 us instead of 368.
+
+// Puts J[0 .. cnt), the slots of the k nearest, in order by (d^2, index) where
+// their entries were equal above the replaced bits (bit m of tied: the m-th and
+// the one after it).  A run of ties that goes on beyond the k-th is chosen from
+// the list first.
+__device__ __forceinline__ void order_ties(float2 p, const float2* __restrict__ pos,
+                                           const uint2* __restrict__ aux, int* raw, int found,
+                                           int* J, int cnt, uint32_t tied, uint32_t replaced) {
+    auto dist2 = [&](int j) {
+        const float2 q = pos[j];
+        return key_d2(p.x, p.y, q.x, q.y);
+    };
+    if ((tied >> (cnt - 1)) & 1u) {
+        const int m = 32 - __clz((int)(~tied & ((1u << (cnt - 1) << 1) - 1u)));
+        const uint32_t run = __float_as_uint(dist2(J[m * 32])) & ~replaced;
+        int members = 0;
+#pragma unroll 4
+        for (int e = 0; e < found; ++e) {
+            const int j = raw[e * 32];
+            if ((__float_as_uint(dist2(j)) & ~replaced) == run) raw[32 * members++] = j;
+        }
+#pragma unroll 1
+        for (int at = m; at < cnt; ++at) {   // the first of those left, each time
+            int best = 0, jb = raw[0], ob = aux_orig(aux[jb]);
+            float db = dist2(jb);
+#pragma unroll 1
+            for (int e = 1; e < members; ++e) {
+                const int j = raw[e * 32];
+                const float d = dist2(j);
+                const int o = aux_orig(aux[j]);
+                if (d < db || (d == db && o < ob)) {
+                    best = e;
+                    jb = j;
+                    db = d;
+                    ob = o;
+                }
+            }
+            J[at * 32] = jb;
+            raw[best * 32] = raw[--members * 32];
+        }
+        tied &= (1u << m) - 1u;
+    }
+#pragma unroll 1
+    for (; tied != 0u; tied &= tied - 1u) {   // insertion sort of every run
+        int at = __ffs((int)tied);            // (the second of the pair)
+        const int j = J[at * 32];
+        const float d = dist2(j);
+        const int o = aux_orig(aux[j]);
+#pragma unroll 1
+        for (; at > 0; --at) {
+            const int i = J[(at - 1) * 32];
+            const float di = dist2(i);
+            if (di < d || (di == d && aux_orig(aux[i]) < o)) break;
+            J[at * 32] = i;
+        }
+        J[at * 32] = j;
+    }
+}
+
+// Grid rows around an agent: its place in them and their lower bounds of dy^2.
+struct Rows {
+    const uint32_t* cs;
+    int cx, cy, nx, ny;
+    float ch, mg, pry, fx;
+};
+
+// The search with a sorted list (slots in J, keys in key and orig), for agents
+// with more candidates at nearly one distance than the list of slots holds.
+__device__ __noinline__ int sorted_search(float2 p, int s, int k, float lim, Rows g,
+                                          const float2* __restrict__ pos,
+                                          const uint2* __restrict__ aux, int* J, float* key,
+                                          int* orig) {
+    int cnt = 0;
+    // candidate j: into the list when before its last entry, the ones behind it shift
+    auto consider = [&](int j, float d2, int oj) {
+        if (!(d2 <= lim) || (cnt == k && d2 == lim && oj > orig[(k - 1) * 32])) return;
+        int at = min(cnt, k - 1);
+        while (at > 0) {
+            const float de = key[(at - 1) * 32];
+            const int oe = orig[(at - 1) * 32];
+            if (de < d2 || (de == d2 && oe < oj)) break;
+            key[at * 32] = de;
+            orig[at * 32] = oe;
+            J[at * 32] = J[(at - 1) * 32];
+            --at;
+        }
+        key[at * 32] = d2;
+        orig[at * 32] = oj;
+        J[at * 32] = j;
+        cnt = min(cnt + 1, k);
+        if (cnt == k) lim = key[(k - 1) * 32];
+    };
+    for (int m = 0;; ++m) {
+        bool any = false;
+        for (int side = m == 0 ? 1 : 0; side < 2; ++side) {
+            const int ry = side == 0 ? g.cy - m : g.cy + m;
+            if (ry < 0 || ry >= g.ny) continue;
+            const float by0 = ry == 0 ? -CUDART_INF_F : (float)ry * g.ch - g.mg;
+            const float by1 = ry == g.ny - 1 ? CUDART_INF_F : (float)(ry + 1) * g.ch + g.mg;
+            const float ey = fmaxf(fmaxf(by0 - g.pry, g.pry - by1), 0.0f);
+            const float g2 = m == 0 ? 0.0f : ey * ey * 0.99999f;
+            if (g2 > lim) continue;
+            any = true;
+            const uint32_t* c = g.cs + (size_t)ry * g.nx;
+            const int rb = (int)c[0], re = (int)c[g.nx];
+            const int b = (int)c[g.cx], e = (int)c[g.cx + 1];
+            int jr = m == 0 ? s + 1 : min(b + (int)(g.fx * (float)(e - b)), e);
+            int jl = m == 0 ? s - 1 : jr - 1;
+            bool ron = jr < re, lon = jl >= rb;
+            while (ron || lon) {
+                float2 qr = p, ql = p;
+                int orr = 0, ol = 0;
+                if (ron) {
+                    qr = pos[jr];
+                    orr = aux_orig(aux[jr]);
+                }
+                if (lon) {
+                    ql = pos[jl];
+                    ol = aux_orig(aux[jl]);
+                }
+                if (ron) {
+                    const float dx = __fsub_rn(qr.x, p.x), dy = __fsub_rn(qr.y, p.y);
+                    const float xx = __fmul_rn(dx, dx);
+                    if (dx > 0.0f && __fadd_rn(xx, g2) > lim) {
+                        ron = false;
+                    } else {
+                        consider(jr, __fadd_rn(xx, __fmul_rn(dy, dy)), orr);
+                        ron = ++jr < re;
+                    }
+                }
+                if (lon) {
+                    const float dx = __fsub_rn(ql.x, p.x), dy = __fsub_rn(ql.y, p.y);
+                    const float xx = __fmul_rn(dx, dx);
+                    if (dx < 0.0f && __fadd_rn(xx, g2) > lim) {
+                        lon = false;
+                    } else {
+                        consider(jl, __fadd_rn(xx, __fmul_rn(dy, dy)), ol);
+                        lon = --jl >= rb;
+                    }
+                }
+            }
+        }
+        if (!any) return cnt;   // both sides at the edge or beyond the bound
+    }
+}
 
 // One thread per agent (sorted slot s), k <= KC, the incremental LP.
 // MODE_PLAIN, or MODE_RECORD with the LP's active set.  kl: line slots per
@@ -92,7 +245,7 @@ agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
         // the largest float below R_n^2: a candidate within the bound (this, or
         // the k-th distance once k are known, its low bits set) is admitted,
         // and a row cursor stops beyond it
-        const float thr0 = R2 > 0.0f ? __int_as_float(__float_as_int(R2) - 1) : -1.0f;
+        float thr0 = R2 > 0.0f ? __int_as_float(__float_as_int(R2) - 1) : -1.0f;
         // sorted; the first KC - k entries are below every distance, the ones
         // not yet found above
         float D[KC + 1];
@@ -109,39 +262,7 @@ agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
         };
         clear();
         const uint32_t* __restrict__ cs = cstart + sc.cell_off;
-        const uint32_t* __restrict__ aux_idx = reinterpret_cast<const uint32_t*>(aux) + 1;
         int found = 0;
-        // whether list entry e comes before candidate (d2, oj)
-        auto before = [&](int e, float d2, int oj) {
-            const int j = raw[e * 32];
-            const float2 q = pos[j];
-            const float de = key_d2(p.x, p.y, q.x, q.y);
-            return de < d2 ||
-                   (de == d2 && aux_orig(make_uint2(0u, __ldg(aux_idx + 2 * j))) < oj);
-        };
-        // make room: keep the entries within the bound; should that not be
-        // enough (many equal distances), the k first by (d^2, index)
-        auto compact = [&](float lim, int room) {
-            int kept = 0;
-            for (int e = 0; e < found; ++e) {
-                const int j = raw[e * 32];
-                const float2 q = pos[j];
-                if (key_d2(p.x, p.y, q.x, q.y) <= lim) raw[32 * kept++] = j;
-            }
-            found = kept;
-            while (found > room && found > k) {   // drop the last by (d^2, index)
-                int last = 0;
-                for (int e = 1; e < found; ++e) {
-                    const int j = raw[e * 32];
-                    const float2 q = pos[j];
-                    if (before(last, key_d2(p.x, p.y, q.x, q.y),
-                               aux_orig(make_uint2(0u, __ldg(aux_idx + 2 * j)))))
-                        last = e;
-                }
-                --found;
-                raw[last * 32] = raw[found * 32];
-            }
-        };
         // Every grid row is one run of slots sorted by x (the binning kernel
         // orders each cell by x, and cells of a row are consecutive in x).
         // A row is scanned outward from the agent's x with two cursors: the
@@ -212,12 +333,27 @@ agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
                 ron = ron && ++jr < re;
                 lon = lon && --jl >= rb;
                 if (found > cap - 2) {
-                    compact(bound(), cap / 2);
+                    // the list is full: the candidates within the bound stay;
+                    // should that be most of them, the search starts again
+                    const float keep = bound();
+                    int kept = 0;
+#pragma unroll 1
+                    for (int e = 0; e < found; ++e) {
+                        const int j = raw[e * 32];
+                        const float2 q = pos[j];
+                        if (key_d2(p.x, p.y, q.x, q.y) <= keep) raw[32 * kept++] = j;
+                    }
+                    found = kept;
                     clear();
+#pragma unroll 1
                     for (int e = 0; e < found; ++e) {
                         const float2 q = pos[raw[e * 32]];
                         insert_pair<KC + 1>(D, entry(key_d2(p.x, p.y, q.x, q.y), e),
                                             CUDART_INF_F);
+                    }
+                    if (found > cap / 2) {
+                        thr0 = -1.0f;   // (nothing is within the bound any more)
+                        ron = lon = false;
                     }
                 }
             }
@@ -248,31 +384,26 @@ agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
             jr = min(b + (int)(fx * (float)(e - b)), e);
             jl = jr - 1;
         }
-        cnt = min(found, k);
-        // the neighbours in order: entry KC - k + m is the m-th, unless entries
-        // that follow one another differ in the replaced bits only
-        const int fill = KC - k;
-        bool tie = false;
+        if (thr0 < 0.0f && R2 > 0.0f) {
+            cnt = sorted_search(p, s, k, __int_as_float(__float_as_int(R2) - 1),
+                                Rows{cs, cx, cy, nx, ny, ch, mg, pry, fx}, pos, aux,
+                                J, reinterpret_cast<float*>(raw), raw + kl * 32);
+        } else {
+            cnt = min(found, k);
+            // the neighbours in order: entry KC - k + m is the m-th, unless entries
+            // that follow one another differ in the replaced bits only
+            const int fill = KC - k;
+            uint32_t tied = 0u;
 #pragma unroll
-        for (int i = 0; i < KC; ++i) {
-            const uint32_t a = __float_as_uint(D[i]), b = __float_as_uint(D[i + 1]);
-            const int at = i - fill;
-            if (at >= 0 && at < cnt) {
-                J[at * 32] = raw[(int)(a & kPlace) * 32];
-                tie |= (a ^ b) <= kPlace && at + 1 < found;
+            for (int i = 0; i < KC; ++i) {
+                const uint32_t a = __float_as_uint(D[i]), b = __float_as_uint(D[i + 1]);
+                const int at = i - fill;
+                if (at >= 0 && at < cnt) {
+                    J[at * 32] = raw[(int)(a & kPlace) * 32];
+                    if ((a ^ b) <= kPlace && at + 1 < found) tied |= 1u << at;
+                }
             }
-        }
-        if (tie) {   // the k first by (d^2, index), in that order
-            compact(bound(), cap);
-            for (int e = 0; e < found; ++e) {
-                const int j = raw[e * 32];
-                const float2 q = pos[j];
-                const float d2 = key_d2(p.x, p.y, q.x, q.y);
-                const int oj = aux_orig(make_uint2(0u, __ldg(aux_idx + 2 * j)));
-                int at = 0;
-                for (int u = 0; u < found; ++u) at += u != e && before(u, d2, oj) ? 1 : 0;
-                if (at < k) J[at * 32] = j;
-            }
+            if (tied != 0u) order_ties(p, pos, aux, raw, found, J, cnt, tied, kPlace);
         }
     }
     __syncwarp(lanes);   // the lines take the place of the lists
