@@ -400,10 +400,12 @@ warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos,
         __syncwarp();
         if (__any_sync(kFull, pass && W.lane[rank] != lane)) {
             __syncwarp();
-            for (int u = 0; u < 32; ++u) {
-                const float e = __shfl_sync(kFull, ds, u);
-                const int ou = __shfl_sync(kFull, oj, u);
-                if (e == ds && ou < oj) ++rank;
+            unsigned same = __match_any_sync(kFull, __float_as_uint(ds)) & ~(1u << lane);
+            if (!pass) same = 0u;
+            while (__any_sync(kFull, same != 0u)) {
+                const int ou = __shfl_sync(kFull, oj, same != 0u ? __ffs((int)same) - 1 : lane);
+                if (same != 0u && ou < oj) ++rank;
+                same &= same - 1u;
             }
             if (pass) W.lane[rank] = lane;
             __syncwarp();
@@ -482,10 +484,16 @@ warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos,
         auto test_loaded = [&](bool on, int j, bool lf, float g2, float2 c, uint32_t oc) {
             float d2 = CUDART_INF_F, dx = 0.0f, dxx = 0.0f;
             if (on) d2 = measure(c, dx, dxx);
-            const unsigned am = __ballot_sync(kFull, on && d2 <= thr_d);
-            if (am != 0u)
-                admit(am, ((unsigned long long)__float_as_uint(d2) << 32) |
-                              (unsigned)aux_orig(make_uint2(0u, oc)), j);
+            const bool cand = on && d2 <= thr_d;
+            if (__ballot_sync(kFull, cand) != 0u) {
+                // (of many at the k-th's distance only those with a smaller index:
+                // 16,000 agents at 16 points 729 -> 211 us a step)
+                const unsigned long long ck = ((unsigned long long)__float_as_uint(d2) << 32) |
+                                              (unsigned)aux_orig(make_uint2(0u, oc));
+                const unsigned long long last = shfl64(key, k - 1);   // (every lane takes part)
+                const unsigned am = __ballot_sync(kFull, cand && ck < last);
+                if (am != 0u) admit(am, ck, j);
+            }
             return !on || ((lf ? dx < 0.0f : dx > 0.0f) && __fadd_rn(dxx, g2) > thr_d);
         };
         auto test = [&](bool on, int j, bool lf, float g2) {
