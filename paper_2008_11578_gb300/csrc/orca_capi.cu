@@ -5,7 +5,7 @@
 // reads the caller's arrays) and one solve kernel (which bins the new positions
 // for the next step where the binning wants it, and writes the last step's
 // results straight into the caller's arrays).  Which of the variants runs depends
-// on the number of agents and on k (solve_by_warp, solve_flat, bin_cluster);
+// on the number of agents and on k (solve_variant, solve_flat, bin_cluster);
 // their results are the same.
 //
 // A single scene and a batch of independent scenes run the same kernels.  A
@@ -250,6 +250,8 @@ cudaError_t prepare_solve(size_t smem, size_t smem_agent) {
     const size_t most_agent = agent_smem(ORCA_MAX_NEIGHBORS, true, kMaxBlock);
     cudaError_t e = cudaSuccess;
     allow_smem(e, solve_kernel<SRC, MODE_COUNT, LP_INCREMENTAL>, smem, most);
+    allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_INCREMENTAL>, smem, most);
+    allow_smem(e, solve_kernel<SRC, MODE_RECORD, LP_INCREMENTAL>, smem, most);
     allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_WORK_UNITS>, smem, most);
     allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_ENUMERATION>, smem, most);
     allow_smem(e, solve_kernel<SRC, MODE_PLAIN, LP_WARP>, smem, most);
@@ -260,7 +262,9 @@ cudaError_t prepare_solve(size_t smem, size_t smem_agent) {
     return e;
 }
 
-// The comparison LP schemes, the counting and the checked variant.
+// The kernel with the sorted list: plain and recording steps of the sizes that
+// solve_variant gives it, the comparison LP schemes, the counting and the checked
+// variant.
 template <class SRC>
 void launch_solve(int mode, int grid, int block, size_t smem, cudaStream_t st, int n, SRC src,
                   const float2* pos, const float2* vel, const uint2* aux, const uint32_t* start,
@@ -270,6 +274,8 @@ void launch_solve(int mode, int grid, int block, size_t smem, cudaStream_t st, i
     solve_kernel<SRC, M, W><<<grid, block, smem, st>>>(n, src, pos, vel, aux, start, ain, vpd, \
                                                         out, dbg, counters, err)
     if (mode == MODE_COUNT) ORCA_SOLVE(MODE_COUNT, LP_INCREMENTAL);
+    else if (mode == MODE_PLAIN) ORCA_SOLVE(MODE_PLAIN, LP_INCREMENTAL);
+    else if (mode == MODE_RECORD) ORCA_SOLVE(MODE_RECORD, LP_INCREMENTAL);
     else if (mode == MODE_WORK_UNITS) ORCA_SOLVE(MODE_PLAIN, LP_WORK_UNITS);
     else if (mode == MODE_ENUMERATION) ORCA_SOLVE(MODE_PLAIN, LP_ENUMERATION);
     else if (mode == MODE_WARP_LP) ORCA_SOLVE(MODE_PLAIN, LP_WARP);
@@ -383,21 +389,34 @@ int step_mode(const Pipeline& P) {
 }
 
 // Largest scene solved with one warp per agent.  One thread per agent takes
-// the length of a thread's serial chain however few agents there are (44 us a
-// launch at 12,000 agents with k = 10, 75 us with k = 16, 254 us at 32,000
-// with k = 32); a warp's chain is 14 us, but the warps of a larger scene queue
-// (2.4 ns an agent with k = 10, 2.7 with 16, 4.1 with 32).  Per thread / per
-// warp: k = 10 at 16,000 agents 44 / 42 us, at 20,000 47 / 49; k = 16 at 24,000
-// 79 / 67, at 32,000 82 / 85; k = 17 at 64,000 176 / 170, at 250,000 553 / 628;
-// k = 20 at 64,000 227 / 186, at 250,000 656 / 686; from k = 24 the warp is
-// ahead at every size (250,000 agents: 797 / 776 us, with k = 32 1143 / 1030).
+// the length of a thread's serial chain however few agents there are; a warp's
+// chain is 14 us, but the warps of a larger scene queue (2.4 ns an agent with
+// k = 10, 2.7 with 16, 4.1 with 32).  Thread / warp, us a launch, moving crowds:
+//   k = 10  16,000 agents 41 / 40, 18,000 42 / 44      k = 12  20,000 50 / 50
+//   k = 16  24,000 70 / 66, 28,000 68 / 70             k = 17  45,000 126 / 120
+//   k = 20  45,000 152 / 128, 64,000 158 / 177         k = 24  90,000 329 / 269
+//   k = 28  131,000 435 / 431                          k = 32  131,000 566 / 499
+// (k <= 16 the register network, up to 25 the sorted list, above the better one).
+// On regular grids, whose agents take like paths, threads are ahead earlier
+// (16,000 agents at rest, k = 10: 27 / 44).
 int warp_solve_max(int k) {
-    return k <= 10 ? 18432 : k <= 16 ? 28672 : k < 24 ? 131072 : INT_MAX;
+    if (k <= 16) return 1664 * std::max(k, 10);
+    return k < 20 ? 47104 : k < 24 ? 57344 : k < 26 ? 102400 : k < 28 ? 122880 : 147456;
 }
 
-bool solve_by_warp(const Pipeline& P, int mode) {
-    return (mode == MODE_PLAIN || mode == MODE_RECORD) && P.kcap <= 32 &&
-           P.n <= warp_solve_max(P.kmax);
+// The kernel of a plain or recording step.  Above the warp's sizes the register
+// network is the faster search up to k = 16 and from k = 26; between, its 33
+// entries cost more than the list's few admissions (network / list, us a launch:
+// k = 17, 260,000 agents 446 / 365, 1M with k = 20 1,846 / 1,535; k = 24 with
+// 131,000 430 / 362, with 260,000 634 / 661; k = 28 538 / 615 at 190,000, k = 32
+// 827 / 1,099 at 260,000).  More than 32 lines (k >= 30 with kinematic limits)
+// always take the network (20,000 agents 138 / 210).
+enum class Solve { warp, network, list };
+
+Solve solve_variant(const Pipeline& P, int mode) {
+    if (mode != MODE_PLAIN && mode != MODE_RECORD) return Solve::list;
+    if (P.kcap <= 32 && P.n <= warp_solve_max(P.kmax)) return Solve::warp;
+    return P.kmax <= 16 || P.kmax >= 26 ? Solve::network : Solve::list;
 }
 
 // Whether the scene is small enough to go without cells, and along which side
@@ -529,7 +548,8 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
     int sb = P.block;
     int sgrid = (n + sb - 1) / sb;
     const size_t smem = solve_smem(P);
-    const bool by_warp = solve_by_warp(P, mode);
+    const Solve variant = solve_variant(P, mode);
+    const bool by_warp = variant == Solve::warp;
     const bool flat = solve_flat(P, by_warp), by_y = flat && flat_by_y(P);
     ClusterShape shape{0, 0, 0};
     const int nb = bin_cluster(P, &shape);
@@ -541,7 +561,7 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
     const bool early = sgrid > 2 * P.bin_grid_max;
     // Grids of several waves end more evenly in blocks of two warps, unless the
     // caller chose the size (1M clusters 375 -> 367 us, 250,000 138 -> 136).
-    if (P.any_block && early && (mode == MODE_PLAIN || mode == MODE_RECORD)) {
+    if (P.any_block && early && variant == Solve::network) {
         sb = 64;
         sgrid = (n + sb - 1) / sb;
     }
@@ -570,11 +590,11 @@ void enqueue_steps(const Pipeline& P, SRC src, int n_steps, const float* vpref_d
         if (by_warp)
             launch_warp_solve(mode, flat, by_y, wgrid, sb, st, n, src, B.pos1, B.vel1,
                               B.aux[cur], B.start, ain, vpd, out, dbg_for(t), B.err);
-        else if (mode == MODE_RECORD)
+        else if (variant == Solve::network && mode == MODE_RECORD)
             launch_agent_solve<SRC, MODE_RECORD>(P.kmax, P.kin, early, sgrid, sb, st, n, src, B.pos1,
                                                  B.vel1, B.aux[cur], B.start, ain, vpd, out,
                                                  dbg_for(t), B.err);
-        else if (mode == MODE_PLAIN)
+        else if (variant == Solve::network)
             launch_agent_solve<SRC, MODE_PLAIN>(P.kmax, P.kin, early, sgrid, sb, st, n, src, B.pos1,
                                                 B.vel1, B.aux[cur], B.start, ain, vpd, out,
                                                 dbg_for(t), B.err);

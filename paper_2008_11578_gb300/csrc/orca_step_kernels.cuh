@@ -634,13 +634,16 @@ __device__ __forceinline__ void limit_lines(const SceneDev& sc, float2 v, float2
 // One thread per agent (sorted slot s).  The neighbour list and then the
 // lines are kept in dynamic shared memory (k float4 slots per thread), slot i
 // of thread t at [i * blockDim.x + t] (conflict-free float4).
-// The search keeps the sorted list itself in shared memory, for the variants
-// that look into it: MODE_COUNT adds work tallies (algorithmic FLOP
-// accounting), MODE_CHECK certifies the results, and LP selects the
-// velocity-LP scheme of MODE_PLAIN, for comparison only: the paper's
-// block-cooperative work units, the warp-cooperative LP (with both, every
-// thread of the block takes part to the end of the LP, lanes past the last
-// agent shadowing it and writing nothing) or active-set enumeration.
+// The search keeps the sorted list itself in shared memory and touches only its
+// entries behind an admitted candidate: ahead of the register network where the
+// list is long and few candidates enter it (solve_variant), and needed by the
+// variants that look into the list.  MODE_COUNT adds work tallies (algorithmic
+// FLOP accounting), MODE_RECORD the LP's active set, MODE_CHECK certifies the
+// results, and LP selects the velocity-LP scheme of MODE_PLAIN: the incremental
+// one, or for comparison only the paper's block-cooperative work units, the
+// warp-cooperative LP (with both, every thread of the block takes part to the
+// end of the LP, lanes past the last agent shadowing it and writing nothing) or
+// active-set enumeration.
 template <class SRC, int MODE, int LP = LP_INCREMENTAL>
 __global__ void __launch_bounds__(128)
 solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* __restrict__ vel,
@@ -921,6 +924,7 @@ solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* __res
             nb[m] = m < cnt ? __float_as_int(L[m * stride].z) : -1;
     }
     bool any_overlap = false;
+    uint32_t capbits = 0u, ovbits = 0u;   // per-line construction (MODE_RECORD)
     for (int i = 0; i < cnt; ++i) {
         const float4 e = L[i * stride];
         const int j = __float_as_int(e.y);
@@ -935,6 +939,10 @@ solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* __res
         bool cap;
         L[i * stride] = orca_line(p.x, p.y, v.x, v.y, r, pj.x, pj.y, vj.x, vj.y, rj, f,
                                   sc.inv_tau, sc.inv_dt, ov, cap);
+        if (MODE == MODE_RECORD) {
+            ovbits |= (ov ? 1u : 0u) << i;
+            capbits |= (cap ? 1u : 0u) << i;
+        }
     }
 
     // ---- vehicles' kinematic half-planes (off unless the scene sets limits) ----
@@ -983,18 +991,33 @@ solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* __res
             }
         }
     }
+    auto nib = [](uint64_t q, int i) { return (uint32_t)((q >> (4 * i)) & 15ull); };
+    auto put = [](uint64_t q, int i, uint32_t x) {
+        return (q & ~(15ull << (4 * i))) | ((uint64_t)x << (4 * i));
+    };
+    uint64_t perm = 0ull;
+    if (MODE == MODE_RECORD && nlines <= 16) {
+        perm = 0xFEDCBA9876543210ull;
+        const uint32_t a0 = nib(perm, sw0);
+        perm = put(put(perm, sw0, nib(perm, 0)), 0, a0);
+        const uint32_t a1 = nib(perm, sw1);
+        perm = put(put(perm, sw1, nib(perm, 1)), 1, a1);
+    }
     if (nlines <= 16) {
         for (int m = 3; m < nlines; ++m) {
             const float4 e = L[m * stride];
             const float pe = penetration(e, v.x, v.y);
+            const uint32_t em = MODE == MODE_RECORD ? nib(perm, m) : 0u;
             int at = m;
             while (at > 2) {
                 const float4 f = L[(at - 1) * stride];
                 if (!(penetration(f, v.x, v.y) < pe)) break;
                 L[at * stride] = f;
+                if (MODE == MODE_RECORD) perm = put(perm, at, nib(perm, at - 1));
                 --at;
             }
             L[at * stride] = e;
+            if (MODE == MODE_RECORD) perm = put(perm, at, em);
         }
     }
 
@@ -1059,6 +1082,24 @@ solve_kernel(int n, SRC src, const float2* __restrict__ pos, const float2* __res
     if (dbg.spos != nullptr) dbg.spos[o] = p;
     if (dbg.svel != nullptr) dbg.svel[o] = v;
     if (dbg.vnew != nullptr) dbg.vnew[o] = make_float2(vx, vy);
+    if (MODE == MODE_RECORD && dbg.act != nullptr) {
+        const int nl = act_nlines(act);
+        for (int m = 0; m < nl; ++m) {
+            // the LP's line index in the neighbour order
+            int li = act_line(act, m);
+            if (nlines <= 16) {
+                li = (int)nib(perm, li);
+            } else {   // undo the two swaps
+                li = li == 1 ? sw1 : (li == sw1 ? 1 : li);
+                li = li == 0 ? sw0 : (li == sw0 ? 0 : li);
+            }
+            act = (act & ~(31u << (8 + 8 * m))) | ((uint32_t)li << (8 + 8 * m));
+            act |= ((capbits >> li) & 1u) << (13 + 8 * m);
+            act |= ((ovbits >> li) & 1u) << (14 + 8 * m);
+        }
+        dbg.act[o] = act;
+    }
+
     if (MODE == MODE_COUNT) {
         const long long end = clock64();
         unsigned long long c[kNumCounters] = {(unsigned long long)n_cand,

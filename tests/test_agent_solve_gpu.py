@@ -117,9 +117,22 @@ def test_many_neighbours_above_the_warp_kernels_limit():
     _both(s, 1)
 
 
+@pytest.mark.parametrize("n,k", [(16640, 10), (16641, 5), (19969, 12), (26625, 16), (47104, 17),
+                                 (47105, 19), (57345, 20), (102401, 25), (122881, 27),
+                                 (147457, 32)])
+def test_around_the_limits(n, k):
+    """On both sides of the sizes at which another solve kernel takes over."""
+    s = scenes.open_square(n, (n / 0.5) ** 0.5, seed=107)
+    s.params.max_neighbors = k
+    rng = np.random.default_rng(5)
+    s.vel = (0.5 * s.max_speed[:, None] * rng.standard_normal((s.n, 2))).astype(np.float32)
+    _both(s, 1)
+
+
 @pytest.mark.parametrize("grid", [False, True])
 @pytest.mark.parametrize("n,k,limits", [(18000, 10, False), (18000, 10, True), (18000, 3, False),
-                                        (28000, 14, True), (28000, 16, False)])
+                                        (28000, 14, True), (28000, 16, False),
+                                        (46000, 17, False), (46000, 19, True)])
 def test_recorded_active_sets(n, k, limits, grid):
     """The same 1,600 agents alone (a warp each) and with n more out of reach."""
     import torch
