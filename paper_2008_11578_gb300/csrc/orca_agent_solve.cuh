@@ -318,8 +318,8 @@ agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
                 const float dyr = __fsub_rn(qr.y, p.y), dyl = __fsub_rn(ql.y, p.y);
                 float dr = __fadd_rn(xxr, __fmul_rn(dyr, dyr));
                 float dl = __fadd_rn(xxl, __fmul_rn(dyl, dyl));
-                if (!ron || dr > lim) dr = CUDART_INF_F;
-                if (!lon || dl > lim) dl = CUDART_INF_F;
+                if (!(ron && dr <= lim)) dr = CUDART_INF_F;   // (not a number either)
+                if (!(lon && dl <= lim)) dl = CUDART_INF_F;
                 float er = dr, el = dl;
                 if (dr < CUDART_INF_F) {
                     er = entry(dr, found);
