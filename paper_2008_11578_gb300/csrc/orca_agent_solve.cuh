@@ -520,16 +520,23 @@ agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
         const uint32_t a1 = nib(perm, sw1);
         perm = put(put(perm, sw1, nib(perm, 1)), 1, a1);
     }
-    if (KC <= 10 && nlines <= 10) {
-        // the rank of each line among slots 2 .. 9, by all pairs (no branches)
-        constexpr int R = 8;
-        float q[R];
-        int at[R];
+    constexpr int R = 8;
+    float q[R];
+    bool by_pairs = KC <= 10 && nlines <= 10;
+    if (by_pairs) {
+        float sum = 0.0f;
 #pragma unroll
         for (int u = 0; u < R; ++u) {
             q[u] = u + 2 < nlines ? pen[(u + 2) * 32] : -CUDART_INF_F;
-            at[u] = 2;
+            sum += q[u];
         }
+        by_pairs = sum == sum;   // (a penetration that is no number has no rank)
+    }
+    if (by_pairs) {
+        // the rank of each line among slots 2 .. 9, by all pairs (no branches)
+        int at[R];
+#pragma unroll
+        for (int u = 0; u < R; ++u) at[u] = 2;
 #pragma unroll
         for (int u = 0; u < R; ++u)
 #pragma unroll
