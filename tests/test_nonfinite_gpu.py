@@ -57,3 +57,23 @@ def test_positions(n, k, limits, axis, value):
     s = _scene(n, k, limits)
     s.pos[::37, axis] = value
     _both(s, 4)
+
+
+@pytest.mark.parametrize("n,k,limits", SIZES)
+@pytest.mark.parametrize("field,value", [("vel", 1e13), ("vel", 1e19), ("vel", 3e38),
+                                         ("vel", np.nan), ("radius", np.nan), ("radius", np.inf),
+                                         ("radius", -1.0), ("max_speed", -5.0),
+                                         ("max_speed", np.inf), ("max_speed", np.nan),
+                                         ("goal", np.inf), ("dt", 1e-20), ("dt", 1e-39)])
+def test_half_planes(n, k, limits, field, value):
+    """Half-planes whose products overflow, or that are no numbers."""
+    s = _scene(n, k, limits)
+    with np.errstate(all="ignore"):
+        if field == "dt":
+            s.params.dt = value
+        elif field == "vel":
+            s.vel[::41] *= np.float32(value)
+        else:
+            getattr(s, field)[::41] = value
+    bad = not np.isfinite(s.vel).all()
+    _both(s, 4 if bad else 0)
