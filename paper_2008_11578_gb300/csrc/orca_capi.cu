@@ -638,6 +638,7 @@ cudaError_t bin_grid_max(int* out) {
 template <class SRC>
 cudaError_t cluster_max(int* out) {
     *out = 0;
+    bool refused = false;
     const size_t smem = (size_t)16 * kClusterSlots + (size_t)4 * kClusterCells + 16;
     for (auto f : {cluster_bin_kernel<SRC, true, kClusterThreads>,
                    cluster_bin_kernel<SRC, false, kClusterThreads>,
@@ -662,17 +663,23 @@ cudaError_t cluster_max(int* out) {
         cfg.numAttrs = 1;
         int k0 = 0, k1 = 0;
         if (cudaOccupancyMaxActiveClusters(&k0, cluster_bin_kernel<SRC, true, kClusterThreads>,
-                                           &cfg) == cudaSuccess &&
+                                           &cfg) != cudaSuccess ||
             cudaOccupancyMaxActiveClusters(&k1, cluster_bin_kernel<SRC, false, kClusterThreads>,
-                                           &cfg) == cudaSuccess &&
-            k0 > 0 && k1 > 0) {
+                                           &cfg) != cudaSuccess) {
+            refused = true;
+        } else if (k0 > 0 && k1 > 0) {
             *out = nb;
             break;
         }
     }
-    cudaGetLastError();   // a size that does not fit is no error of the caller's
+    if (refused) cudaGetLastError();   // a size that does not fit is no error of the caller's
     return cudaSuccess;
 }
+
+// An error that the caller has pending with the runtime when it steps is reported
+// by the step (cudaGetLastError after the launches); cudaFuncSetAttribute clears
+// it, so the calls that prepare and step in one look before.
+bool error_pending() { return cudaPeekAtLastError() != cudaSuccess; }
 
 int prepare(Pipeline& P) {
     const size_t smem = solve_smem(P);
@@ -725,6 +732,7 @@ void drop_graph(Pipeline& P) {
 int capture_graph(Pipeline& P, int n_steps, const float* vpref_delta) {
     drop_graph(P);
     if (P.n == 0 || n_steps == 0) return ORCA_OK;
+    const bool pending = error_pending();
     int st = prepare(P);
     if (st != ORCA_OK) return st;
     cudaStream_t cs = nullptr;
@@ -737,6 +745,7 @@ int capture_graph(Pipeline& P, int n_steps, const float* vpref_delta) {
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         st = run_steps(P, n_steps, vpref_delta, cs);
+        if (st == ORCA_OK && pending) st = ORCA_ERR_CUDA;
         e = cudaStreamEndCapture(cs, &g);
         if (st == ORCA_OK && e == cudaSuccess) e = cudaGraphInstantiate(&P.graph, g, 0);
     }
@@ -1499,6 +1508,7 @@ extern "C" int orca_step_noalloc(const orca_params* params, const orca_agents* a
                   params->block_size,
                   0, L, w, params->max_neighbors, params->debug_flags);
     P.one = scene_dev(params, 0, n, 0);
+    const bool pending = error_pending();
     st = prepare(P);
     if (st != ORCA_OK) return st;
     // the error word, the barrier words and the cell counts start at zero
@@ -1506,6 +1516,7 @@ extern "C" int orca_step_noalloc(const orca_params* params, const orca_agents* a
         cudaMemsetAsync(P.buf.count, 0, ncells * 4, stm) != cudaSuccess)
         return ORCA_ERR_CUDA;
     st = run_steps(P, n_steps, vpref_delta, stm);
+    if (st == ORCA_OK && pending) st = ORCA_ERR_CUDA;
     if (st != ORCA_OK) return st;
     if (synchronize) {
         if (cudaStreamSynchronize(stm) != cudaSuccess) return ORCA_ERR_CUDA;
