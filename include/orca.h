@@ -286,7 +286,7 @@ int orca_scene_graph_launch(orca_scene *scene, void *stream);
  * Synchronise the device, then read and clear the scene's device error
  * word.  Returns ORCA_OK or the first recorded error status.
  * ORCA_ERR_TIMEOUT: a grid barrier of the binning kernel waited longer than
- * about half a second, or a later step found the cell counts such a step
+ * about a second, or a later step found the cell counts such a step
  * left behind (or two calls ran on one scene at once); the results of those
  * steps are invalid.  This call also resets the barrier and the cell counts,
  * so the scene can step again.

@@ -71,7 +71,7 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* warp_s
 //      and moves its agent's state there.
 // Later steps skip A: the solve kernel bins the new positions as it writes
 // them.  Grid barriers separate the phases.  The cooperative launch keeps
-// every block resident; a barrier that waits longer than about half a second
+// every block resident; a barrier that waits longer than about a second
 // flags ERR_BIT_TIMEOUT and every block leaves the kernel.
 // The cell counts are zero on entry: the workspace is cleared once when a
 // scene is created, and phase C clears them again every step.  Should they
@@ -85,7 +85,7 @@ constexpr int kRankPerThread = 4;    // slots per thread and chunk in E
 constexpr int kRankChunk = kBinThreads * kRankPerThread;
 constexpr int kRankHalo = 128;       // keys staged on either side of a chunk in E
 constexpr int kBinGridMax = 4096;    // launch blocks at most (block-sum slots)
-constexpr unsigned kBarrierSpins = 1u << 20;   // about half a second
+constexpr unsigned kBarrierSpins = 1u << 22;   // about a second (0.22 us a poll)
 
 struct BinArgs {
     int n, ncells;
