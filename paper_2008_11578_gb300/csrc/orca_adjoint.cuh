@@ -266,10 +266,10 @@ __device__ __forceinline__ float2 ld_after_wait(const float2* p) {
 // runs, and the wait stands before the first cotangent and before every write
 // (4,064 agents, 16 steps and their gradient 648 -> 612 us, 2.2 us a launch).
 __global__ void __launch_bounds__(128)
-adjoint_kernel(int n, SceneDev sc, const float2* __restrict__ pos, const float2* __restrict__ vel,
+adjoint_kernel(int n, SceneDev sc, const float2* pos, const float2* vel,
                const float* __restrict__ rad, const uint8_t* __restrict__ typ,
-               const int32_t* __restrict__ nbr, int k_stride, const uint32_t* __restrict__ act,
-               const uint8_t* __restrict__ wp_used, const float2* __restrict__ vnew, AgentIn ain,
+               const int32_t* nbr, int k_stride, const uint32_t* act, const uint8_t* wp_used,
+               const float2* vnew, AgentIn ain,
                const float2* __restrict__ vpd, const float2* pbar_next,
                const float2* vbar_next, const float2* __restrict__ dl_dv,
                float2* __restrict__ pbar_cur, float2* __restrict__ vbar_cur,

@@ -61,8 +61,7 @@ __host__ __device__ constexpr int agent_units(int kl) { return kl + (kl + 3) / 4
 // their entries were equal above the replaced bits (bit m of tied: the m-th and
 // the one after it).  A run of ties that goes on beyond the k-th is chosen from
 // the list first.
-__device__ __forceinline__ void order_ties(float2 p, const float2* __restrict__ pos,
-                                           const uint2* __restrict__ aux, int* raw, int found,
+__device__ __forceinline__ void order_ties(float2 p, const float2* pos, const uint2* aux, int* raw, int found,
                                            int* J, int cnt, uint32_t tied, uint32_t replaced) {
     auto dist2 = [&](int j) {
         const float2 q = pos[j];
@@ -125,8 +124,7 @@ struct Rows {
 // The search with a sorted list (slots in J, keys in key and orig), for agents
 // with more candidates at nearly one distance than the list of slots holds.
 __device__ __noinline__ int sorted_search(float2 p, int s, int k, float lim, Rows g,
-                                          const float2* __restrict__ pos,
-                                          const uint2* __restrict__ aux, int* J, float* key,
+                                          const float2* pos, const uint2* aux, int* J, float* key,
                                           int* orig) {
     int cnt = 0;
     // candidate j: into the list when before its last entry, the ones behind it shift
@@ -207,9 +205,8 @@ __device__ __noinline__ int sorted_search(float2 p, int s, int k, float lim, Row
 // lane (KC, and the kinematic half-planes if the scene has them).
 template <class SRC, int MODE, int KC>
 __global__ void __launch_bounds__(128, KC <= 10 ? 7 : 1)
-agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
-                   const float2* __restrict__ vel, const uint2* __restrict__ aux,
-                   const uint32_t* __restrict__ cstart, AgentIn ain,
+agent_solve_kernel(int n, int kl, SRC src, const float2* pos, const float2* vel,
+                   const uint2* aux, const uint32_t* cstart, AgentIn ain,
                    const float2* __restrict__ vpd, StepOut out, DebugOut dbg,
                    int* __restrict__ err) {
     extern __shared__ float4 smem_lines[];
@@ -261,7 +258,7 @@ agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
             return __uint_as_float((__float_as_uint(d2) & ~kPlace) | (uint32_t)place);
         };
         clear();
-        const uint32_t* __restrict__ cs = cstart + sc.cell_off;
+        const uint32_t* cs = cstart + sc.cell_off;
         int found = 0;
         // Every grid row is one run of slots sorted by x (the binning kernel
         // orders each cell by x, and cells of a row are consecutive in x).
@@ -303,7 +300,7 @@ agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
         int ry = cy, jr = s + 1, jl = s - 1;
         float g2 = 0.0f;
         for (;;) {
-            const int rb = (int)__ldg(cs + ry * nx), re = (int)__ldg(cs + ry * nx + nx);
+            const int rb = (int)cs[ry * nx], re = (int)cs[ry * nx + nx];
             bool ron = jr < re, lon = jl >= rb;
             float2 nr = pos[min(jr, n - 1)], nl = pos[max(jl, 0)];
             while (ron || lon) {
@@ -380,7 +377,7 @@ agent_solve_kernel(int n, int kl, SRC src, const float2* __restrict__ pos,
             }
             if (!more) break;
             const int c = ry * nx + cx;
-            const int b = (int)__ldg(cs + c), e = (int)__ldg(cs + c + 1);
+            const int b = (int)cs[c], e = (int)cs[c + 1];
             jr = min(b + (int)(fx * (float)(e - b)), e);
             jl = jr - 1;
         }

@@ -75,7 +75,7 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     // ---- the agents of this block and their cells ----
     // (first step: in the order that the previous call recorded, if it did, so
     // that a block's agents lie in few blocks' cells)
-    const uint32_t* __restrict__ hint = nullptr;
+    const uint32_t* hint = nullptr;
     if (FIRST && __ldcg(a.err + 1) != 0) hint = a.hint;
     const int i0 = r << sh.slot_shift;
     const int iend = min(i0 + sn, a.n);
@@ -87,7 +87,7 @@ cluster_bin_kernel(SRC src, BinArgs a, ClusterShape sh) {
     for (int u = 0; u < kClusterPerThread; ++u) {
         from[u] = i0 + tid + u * NT;
         if (FIRST && hint != nullptr && from[u] < iend) {
-            const uint32_t h = __ldg(hint + from[u]);
+            const uint32_t h = hint[from[u]];
             if (h < (uint32_t)a.n) from[u] = (int)h;
             else lost = true;
         }
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kFlatThreads) flat_bin_kernel(BinArgs a, bool 
     __shared__ uint32_t keys[kFlatMax];
     launch_dependents();
     wait_for_primary();
-    const float2* __restrict__ pos = FIRST ? a.upos : a.pos0;
+    const float2* pos = FIRST ? a.upos : a.pos0;
     const int tid = (int)threadIdx.x, q = tid % kFlatLanes;
     const int i = (int)blockIdx.x * kFlatAgents + tid / kFlatLanes;
     float2 p = make_float2(0.0f, 0.0f), v = p;

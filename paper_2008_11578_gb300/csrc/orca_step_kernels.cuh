@@ -19,7 +19,9 @@ namespace orca {
 // kernel before them still runs, once all its blocks have called
 // launch_dependents() (or exited); wait_for_primary() returns when that
 // kernel has finished and its writes are visible.  Without the launch
-// attribute both do nothing.
+// attribute both do nothing.  What the kernel before writes is read after the
+// wait through plain pointers: const __restrict__ and __ldg promise that the data
+// does not change while the kernel runs, and let the load move ahead of the wait.
 __device__ __forceinline__ void launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
@@ -89,13 +91,13 @@ constexpr unsigned kBarrierSpins = 1u << 22;   // about a second (0.22 us a poll
 
 struct BinArgs {
     int n, ncells;
-    const float2* __restrict__ upos;   // caller arrays, caller order (first step)
-    const float2* __restrict__ uvel;
+    const float2* upos;   // caller arrays, caller order (first step)
+    const float2* uvel;
     const float* __restrict__ urad;
     const uint8_t* __restrict__ utype;
-    const float2* __restrict__ pos0;   // the previous solve's output (later steps)
-    const float2* __restrict__ vel0;
-    const uint2* __restrict__ aux0;
+    const float2* pos0;   // the previous solve's output (later steps)
+    const float2* vel0;
+    const uint2* aux0;
     float2* __restrict__ stage_pos;    // first step: the caller's state in binning order
     float2* __restrict__ stage_vel;
     uint2* __restrict__ stage_aux;
@@ -109,7 +111,7 @@ struct BinArgs {
     float2* __restrict__ vel1;
     uint2* __restrict__ aux1;
     int* __restrict__ err;             // [0] status bits, [1] hint valid, [2] the grid barrier
-    const uint32_t* __restrict__ hint; // first step: original index per previous sorted slot
+    const uint32_t* hint;              // first step: original index per previous sorted slot
     int test_skip_arrival;             // ORCA_DEBUG_BARRIER_TIMEOUT
 };
 

@@ -337,9 +337,8 @@ __device__ __noinline__ void finish_by_one_lane(WarpSlots& W, int n, float vmax,
 // while the ones before are tested.
 template <class SRC, int MODE, bool FLAT>
 __global__ void __launch_bounds__(128, 8)
-warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos,
-                  const float2* __restrict__ vel, const uint2* __restrict__ aux,
-                  const uint32_t* __restrict__ cstart, AgentIn ain,
+warp_solve_kernel(int n, bool by_y, SRC src, const float2* pos, const float2* vel,
+                  const uint2* aux, const uint32_t* cstart, AgentIn ain,
                   const float2* __restrict__ vpd, StepOut out, DebugOut dbg,
                   int* __restrict__ err) {
     __shared__ WarpSlots slots[4];
@@ -387,10 +386,9 @@ warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos,
     unsigned long long key = ~0ull;
     int slot = -1, cnt = 0;
     if (k > 0 && isfinite(p.x) && isfinite(p.y)) {
-        const uint32_t* __restrict__ aux_idx = reinterpret_cast<const uint32_t*>(aux) + 1;
         const float R2 = sc.R2;
         const float thr0 = R2 > 0.0f ? __int_as_float(__float_as_int(R2) - 1) : -1.0f;
-        const uint32_t* __restrict__ cs = cstart + sc.cell_off;
+        const uint32_t* cs = cstart + sc.cell_off;
         const int nx = sc.nx, ny = sc.ny;
         const float ch = sc.cell_h, mg = sc.ring_delta * ch;
         const float pry = __fsub_rn(p.y, sc.origin_y);
@@ -411,7 +409,7 @@ warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos,
             const int ry = row0 + (lane >> 2), q = lane & 3;
             range = 0;
             if (ry >= 0 && ry < ny)
-                range = (int)__ldg(cs + (size_t)ry * nx + (q == 0 ? 0 : q == 1 ? nx : cx + q - 2));
+                range = (int)cs[(size_t)ry * nx + (q == 0 ? 0 : q == 1 ? nx : cx + q - 2)];
         };
         if (!FLAT) load_rows();
         // ---- seed ----
@@ -424,7 +422,7 @@ warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos,
         auto load = [&](int j, float2& c, uint32_t& oc) {
             if (j >= 0 && j < n) {
                 c = pos[j];
-                oc = __ldg(aux_idx + 2 * j);
+                oc = aux[j].y;
             }
         };
         if (FLAT) {
@@ -479,7 +477,7 @@ warp_solve_kernel(int n, bool by_y, SRC src, const float2* __restrict__ pos,
         float ds = CUDART_INF_F, dxs = 0.0f, dxxs = 0.0f;
         uint32_t os = 0u;
         if (in) {
-            os = __ldg(aux_idx + 2 * js);
+            os = aux[js].y;
             const float d2 = measure(pos[js], dxs, dxxs);
             if (d2 <= thr0) ds = d2;
         }
