@@ -21,7 +21,8 @@
 // ranks the admitted slots, 394 with the places carried in the entries, 378 with
 // the LP's order by all pairs and the penetrations kept for the LP (the
 // 65,000-agent shared space: 67, 55, 58, 52), 375 with one construction of the
-// cut-off and overlap half-planes, 367 in blocks of two warps.  (The benchmark's
+// cut-off and overlap half-planes, 367 in blocks of two warps, 376 with the sorted
+// state read through plain pointers (see wait_for_primary).  (The benchmark's
 // 1M crowd after its warm-up steps: 381 -> 304 us.)  Of the 378 the row scan took
 // about 90 us, the network 60, the half-planes 58, the LP 130.  Registers, in the
 // same form: seven blocks of four warps an SM (72) 380 us and 73 us at 130,000

@@ -434,7 +434,8 @@ bool flat_by_y(const Pipeline& P) {
 }
 
 // Largest scene binned by a cluster.  Against bin_kernel (first step of a call
-// / later steps): 1,000 agents 18 / 14 us -> 14 / 10 us, 16,000 agents
+// / later steps): 1,000 agents (a batch of that size: a single scene goes without
+// cells) 18 / 14 us -> 14 / 10 us, 16,000 agents
 // 22 / 16 -> 15 / 12 us, 32,000 agents 23 / 16 -> 20 / 14 us; a scene's very
 // first step, in the caller's order, 26 -> 16 us at 1,000, 25 -> 23 us at 16,000
 // and 26 -> 32 us at 32,000, where the 16 SMs of the cluster fall behind.

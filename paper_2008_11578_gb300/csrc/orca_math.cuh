@@ -3,7 +3,10 @@
 // Discrete decisions (cell, neighbour key, overlap, waypoint advance, leg
 // side) use explicitly rounded intrinsics in a fixed order so that they
 // never get contracted into FMAs: they are part of the specification both
-// implementations evaluate identically.  Everything else is plain FP32.
+// implementations evaluate identically.  The half-planes and the velocity LPs
+// are FP32 with every contraction written out (mul_add), so that all solve
+// kernels give the same bits; only the comparison LP schemes leave it to the
+// compiler.
 #pragma once
 
 #include <cuda_runtime.h>

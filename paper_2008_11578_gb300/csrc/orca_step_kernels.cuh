@@ -2,10 +2,11 @@
 //
 // Here: the binning kernel of larger scenes (one cooperative launch per step,
 // a counting sort by cell in five phases), the removal of arrived agents, the
-// pieces of a step that all solve kernels share, and the solve kernel of the
-// counting, checked and comparison variants.  Small scenes are binned by
-// orca_cluster_bin.cuh; plain and recording steps are solved by
-// orca_warp_solve.cuh (small scenes) and orca_agent_solve.cuh.  The solve
+// pieces of a step that all solve kernels share, and the solve kernel with the
+// sorted list: large scenes with k = 17 to 25, and the counting, checked and
+// comparison variants.  Small scenes are binned by orca_cluster_bin.cuh; other
+// plain and recording steps are solved by orca_warp_solve.cuh (small scenes) and
+// orca_agent_solve.cuh.  The solve
 // kernels take the agents in cell-sorted order, so the agents of a block come
 // from a few neighbouring cells and read the same candidates through L1.
 #pragma once

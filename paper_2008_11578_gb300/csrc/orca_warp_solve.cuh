@@ -9,11 +9,12 @@
 //                next violated line is found by a vote, not by a loop
 // Every expression and every discrete choice is the per-thread kernel's
 // (agent_solve_kernel), so a step's results do not depend on which one ran.
-// Bound by the latency of one agent's chain while the scene is small (1,000
-// agents: 51 -> 14 us a launch, about 12,500 cycles an agent: loads 1,600,
-// seed 2,100, scan 1,900, half-planes 1,400, order 900, LP 3,600), then by
-// issue slots (16,000 agents: 51 -> 39.5 us, 73 % of issue slots busy; eight
-// blocks an SM 39.7 us, seven 40.9, six 41.0, five 43.0).
+// Bound by the latency of one agent's chain while the scene is small (4,000
+// agents: 49 -> 17 us a launch; with cells, as in a batch, 1,000 agents take 14 us,
+// about 12,500 cycles an agent: loads 1,600, seed 2,100, scan 1,900, half-planes
+// 1,400, order 900, LP 3,600), then by issue slots (16,000 agents: 51 -> 40 us,
+// 73 % of issue slots busy; eight blocks an SM 39.7 us, seven 40.9, six 41.0,
+// five 43.0).
 #pragma once
 
 #include "orca_step_kernels.cuh"
